@@ -807,7 +807,7 @@ __global__ void __launch_bounds__(kEThreads) k_eta_stencil(const __grid_constant
 }
 
 // ---------------------------------------------------------------------------
-// K2: transform along x2, in place; tiles of y_w modes x n2 rows x n_c
+// K2 (3D): transform along x2, in place; tiles of y_w modes x n2 rows x n_c
 // ---------------------------------------------------------------------------
 // W: modes per tile (a compile-time tile geometry; the last tile along x1 may
 // hold fewer modes, its other columns are transformed but never stored).
@@ -1163,13 +1163,18 @@ __device__ __forceinline__ void k_fourier_z_body(const IterArgs<T>& a, const Axi
   typedef typename Cplx<T>::type T2;
   constexpr int NC = Comp<DIM>::NC;
   constexpr int NT = strided_threads(W);
+  // The last transformed axis: x3, or x2 in 2D, where this pass is the whole strided work of the
+  // iteration (x2 transform, Fourier-space work, inverse x2 transform) on tiles of x2 rows.  (As an x3
+  // pass with n3 = 1 between two x2 passes, a block had one row of at most 16 modes for its 256
+  // threads: 512^2 FP64, G^R accelerated, 542 -> 245 us per iteration; 128^2, direct, 63 -> 44 us.)
+  constexpr int AX = DIM - 1;
   if (a.ctrl->state != kRunning) return;
   const Geom g = a.g;
-  const int n3 = g.n3;
+  const int nl = DIM == 3 ? g.n3 : g.n2;
   T2* tile;
-  const T2* tws = load_twiddles(a.tw[2], n3, kTwStrided, &tile);
+  const T2* tws = load_twiddles(a.tw[AX], nl, kTwStrided, &tile);
   const int x0 = blockIdx.x * W;
-  const int py = blockIdx.y;
+  const int py = DIM == 3 ? blockIdx.y : 0;
   const bool do_green = kind == 0;
   const bool do_eta = !a.eta_real && (a.dual ? (kind == 1) : true);
   const int nx = min(W, g.H - x0);
@@ -1177,9 +1182,9 @@ __device__ __forceinline__ void k_fourier_z_body(const IterArgs<T>& a, const Axi
   const int cols = nx * NC;
   T2* spec = kind ? a.specB : a.specA;
   const long long base = ((long long)py * g.H + x0) * NC;
-  const long long zstride = (long long)g.n2 * g.H * NC;
-  if (!tile_load<C, true>(tile, spec + base, zstride, n3, cols, a.ctrl)) return;
-  tile_fft_strided<C, NT, false, false>(tile, pl[2], tws);
+  const long long zstride = (DIM == 3 ? (long long)g.n2 : 1LL) * g.H * NC;
+  if (!tile_load<C, true>(tile, spec + base, zstride, nl, cols, a.ctrl)) return;
+  tile_fft_strided<C, NT, false, false>(tile, pl[AX], tws);
   T eta_acc = (T)0;
   if constexpr (FAST) {
     static_assert(DIM == 3 && NT % W == 0, "fast Fourier pass: 3D, whole modes per thread");
@@ -1190,7 +1195,7 @@ __device__ __forceinline__ void k_fourier_z_body(const IterArgs<T>& a, const Axi
       const T c0 = (T)((a.lam0 + a.mu0) / (a.lam0 + 2.0 * a.mu0));
       const T bxy = rx.y * ry.y, axy = rx.x * ry.y, bxay = rx.y * ry.x;
       const bool line0 = (x0 + xc == 0) && (py == 0);
-      for (int pz = (int)threadIdx.x / W; pz < n3; pz += NT / W) {
+      for (int pz = (int)threadIdx.x / W; pz < nl; pz += NT / W) {
         const T2 rz = __ldg(&a.rd[2][pz]);
         T2* mp = tile + pz * C + xc * NC;
         T2 X[6];
@@ -1206,10 +1211,11 @@ __device__ __forceinline__ void k_fourier_z_body(const IterArgs<T>& a, const Axi
   } else {
     FastDiv fnx = {0u, 0u, 1};  // full tiles (nx == W) divide by the compile-time width
     if (nx != W) fnx = make_fastdiv(nx);
-    const int ym = __ldg(&a.perm[1][py]);
-    for (int idx = threadIdx.x; idx < n3 * nx; idx += blockDim.x) {
+    const int ym3 = DIM == 3 ? __ldg(&a.perm[1][py]) : 0;
+    for (int idx = threadIdx.x; idx < nl * nx; idx += blockDim.x) {
       const int pz = nx == W ? (int)((unsigned)idx / W) : fdiv(idx, fnx), xc = idx - pz * nx;
-      const int zm = __ldg(&a.perm[2][pz]);
+      const int lm = __ldg(&a.perm[AX][pz]);
+      const int ym = DIM == 3 ? ym3 : lm, zm = DIM == 3 ? lm : 0;
       T2* mp = tile + pz * C + xc * NC;
       T2 X[NC];
 #pragma unroll
@@ -1225,8 +1231,8 @@ __device__ __forceinline__ void k_fourier_z_body(const IterArgs<T>& a, const Axi
   }
   __syncthreads();
   if (do_green) {
-    tile_fft_strided<C, NT, true, false>(tile, pl[2], tws);
-    tile_store<C, true>(tile, spec + base, zstride, n3, cols);
+    tile_fft_strided<C, NT, true, false>(tile, pl[AX], tws);
+    tile_store<C, true>(tile, spec + base, zstride, nl, cols);
   }
   if (!a.eta_real) {  // with the real-space eta the x1 pass owns part_eta
     double e1[1] = {(double)eta_acc};
@@ -1705,7 +1711,7 @@ cudaError_t launch_eta_stencil_t(const IterArgs<T>& a, cudaStream_t s) {
 
 template <typename T, bool GRP>
 cudaError_t launch_mid_y_t(const IterArgs<T>& a, bool inv, cudaStream_t s) {
-  if (a.g.n2 == 1) return cudaSuccess;
+  if (a.dim == 2 || a.g.n2 == 1) return cudaSuccess;  // 2D: the Fourier pass transforms along x2
   dim3 grid((a.g.H + a.y_w - 1) / a.y_w, a.g.n3, ((!inv && a.dual && !a.eta_real) ? 2 : 1) * (GRP ? a.nsmp : 1));
 #define FFTLS_MIDY(NCV, WV) k_mid_y<T, NCV, WV, GRP><<<grid, strided_threads(WV), a.y_smem, s>>>(a, inv ? 1 : 0)
 #define FFTLS_MIDY_W(NCV)                                                                               \
@@ -1717,9 +1723,7 @@ cudaError_t launch_mid_y_t(const IterArgs<T>& a, bool inv, cudaStream_t s) {
     case 16: FFTLS_MIDY(NCV, 16); break;                                                                \
     default: return cudaErrorInvalidValue;                                                              \
   }
-  if (a.dim == 3) { FFTLS_MIDY_W(6) }
-  else if constexpr (!GRP) { FFTLS_MIDY_W(3) }
-  else return cudaErrorInvalidValue;
+  FFTLS_MIDY_W(6)
 #undef FFTLS_MIDY_W
 #undef FFTLS_MIDY
   return cudaGetLastError();
@@ -1733,7 +1737,7 @@ bool fourier_fast(const IterArgs<T>& a) {
 
 template <typename T, bool GRP>
 cudaError_t launch_fourier_z_t(const IterArgs<T>& a, cudaStream_t s) {
-  dim3 grid((a.g.H + a.z_w - 1) / a.z_w, a.g.n2, ((a.dual && !a.eta_real) ? 2 : 1) * (GRP ? a.nsmp : 1));
+  dim3 grid((a.g.H + a.z_w - 1) / a.z_w, a.dim == 3 ? a.g.n2 : 1, ((a.dual && !a.eta_real) ? 2 : 1) * (GRP ? a.nsmp : 1));
 #define FFTLS_FZ(D, WV, F) k_fourier_z<T, D, WV, F, GRP><<<grid, strided_threads(WV), a.z_smem, s>>>(a)
 #define FFTLS_FZ_W(D, F)                                                                                \
   switch (a.z_w) {                                                                                      \
@@ -1759,7 +1763,8 @@ cudaError_t launch_fourier_z_t(const IterArgs<T>& a, cudaStream_t s) {
 
 template <typename T, bool GRP>
 cudaError_t launch_reduce_eta_t(const IterArgs<T>& a, cudaStream_t s) {
-  const int nparts = a.eta_real ? a.e_blocks : ((a.g.H + a.z_w - 1) / a.z_w) * a.g.n2 * (a.dual ? 2 : 1);
+  const int nparts = a.eta_real ? a.e_blocks
+                                : ((a.g.H + a.z_w - 1) / a.z_w) * (a.dim == 3 ? a.g.n2 : 1) * (a.dual ? 2 : 1);
   const int mparts = a.x1_blocks;
   const dim3 grid(1, GRP ? a.nsmp : 1);
   if (a.dim == 3) k_reduce_eta<T, 3, GRP><<<grid, kRedThreads, 0, s>>>(a, nparts, mparts);
@@ -1814,13 +1819,6 @@ cudaError_t set_attrs_y_t(size_t smax) {
   FFTLS_ATTR((k_mid_y<T, 6, 4, GRP>));
   FFTLS_ATTR((k_mid_y<T, 6, 8, GRP>));
   FFTLS_ATTR((k_mid_y<T, 6, 16, GRP>));
-  if constexpr (!GRP) {
-    FFTLS_ATTR((k_mid_y<T, 3, 1, GRP>));
-    FFTLS_ATTR((k_mid_y<T, 3, 2, GRP>));
-    FFTLS_ATTR((k_mid_y<T, 3, 4, GRP>));
-    FFTLS_ATTR((k_mid_y<T, 3, 8, GRP>));
-    FFTLS_ATTR((k_mid_y<T, 3, 16, GRP>));
-  }
   return e;
 }
 

@@ -483,11 +483,12 @@ bool apply_plan(const Setup& S, IterArgs<T>& a, bool real_eta, const TilePlan& P
   a.x_threads = 256;
   a.x1_blocks = (int)std::min<long long>((G.nlines + G1 - 1) / G1, (long long)S.num_sms * 8);
   a.x5_blocks = (int)std::min<long long>((G.nlines + G5 - 1) / G5, (long long)S.num_sms * 8);
-  a.y_smem = strided_smem(g.n2, P.y_w, S.nc, sizeof(T2));
-  a.z_smem = strided_smem(g.n3, P.z_w, S.nc, sizeof(T2));
-  if (a.y_smem > G.lim || a.z_smem > G.lim) return false;
+  // 2D: the Fourier pass works on x2 tiles (the x2 pass's width) and the x2 pass does not run
   a.y_w = P.y_w;
-  a.z_w = P.z_w;
+  a.z_w = S.dim == 3 ? P.z_w : P.y_w;
+  a.y_smem = strided_smem(g.n2, a.y_w, S.nc, sizeof(T2));
+  a.z_smem = S.dim == 3 ? strided_smem(g.n3, a.z_w, S.nc, sizeof(T2)) : a.y_smem;
+  if (a.y_smem > G.lim || a.z_smem > G.lim) return false;
   a.y_threads = fftls::strided_threads(a.y_w);
   a.z_threads = fftls::strided_threads(a.z_w);
   a.e_planes = a.e_blocks = 0;
@@ -520,11 +521,12 @@ struct Runner {
   Ctrl* hctl;          // their control blocks on the host (pinned), read after every chunk
   Runner(fftls_ctx* c_, const Setup& S_) : c(c_), S(S_), hctl(c_->h_ctrl) { memset(&a, 0, sizeof(a)); }
 
-  int kernels_per_iter() const { return 4 + (S.g.n2 > 1 ? 2 : 0) + (a.want_delta ? 1 : 0) + (a.eta_real ? 1 : 0); }
+  bool has_mid_y() const { return S.dim == 3 && S.g.n2 > 1; }
+  int kernels_per_iter() const { return 4 + (has_mid_y() ? 2 : 0) + (a.want_delta ? 1 : 0) + (a.eta_real ? 1 : 0); }
 
   fftls_status launch(int kind, cudaError_t (*fn)(Runner*, cudaStream_t), bool prof) {
     const int pi = Prec<T>::idx;
-    if (!capturing) c->launches += (kind == 1 || kind == 4) ? (S.g.n2 > 1) : 1;
+    if (!capturing) c->launches += (kind == 1 || kind == 4) ? has_mid_y() : 1;
     if (prof) {
       cudaEvent_t e0, e1;
       cudaEventCreate(&e0);
@@ -787,11 +789,15 @@ fftls_status tune_plan(fftls_ctx* c, const Setup& S, IterArgs<T>& a, bool real_e
     P.*tf = bt;
     apply_plan<T>(S, a, real_eta, P);
   };
-  if (S.g.n2 > 1)
-    search_wt(&TilePlan::y_w, &TilePlan::y_thr,
-              [](const IterArgs<T>& x, cudaStream_t st) { return launch_mid_y<T>(x, false, st); });
-  search_wt(&TilePlan::z_w, &TilePlan::z_thr,
-            [](const IterArgs<T>& x, cudaStream_t st) { return launch_fourier_z<T>(x, st); });
+  const LaunchFn fourier = [](const IterArgs<T>& x, cudaStream_t st) { return launch_fourier_z<T>(x, st); };
+  if (S.dim == 2)
+    search_wt(&TilePlan::y_w, &TilePlan::y_thr, fourier);
+  else {
+    if (S.g.n2 > 1)
+      search_wt(&TilePlan::y_w, &TilePlan::y_thr,
+                [](const IterArgs<T>& x, cudaStream_t st) { return launch_mid_y<T>(x, false, st); });
+    search_wt(&TilePlan::z_w, &TilePlan::z_thr, fourier);
+  }
   a.eps = (T*)c->specB.p;  // scratch target of the inverse pass's update
   // inverse x1 pass: lines per batch and (FP32) eps loaded by the threads or staged by bulk copies, jointly
   {
@@ -1741,7 +1747,7 @@ extern "C" fftls_status fftls_solve_noalloc(const fftls_problem* p, const fftls_
   const size_t o_specA = take((size_t)S.g.modes * nc * 16);
   const size_t o_specB = take((size_t)S.g.modes * nc * 16);
   const size_t o_pmean = take((size_t)std::max(a.x1_blocks, sblocks) * 2 * nc * 8);
-  const size_t o_peta = take((size_t)ntz * S.g.n2 * 2 * 8);
+  const size_t o_peta = take((size_t)ntz * (d == 3 ? S.g.n2 : 1) * 2 * 8);
   const size_t o_pdelta = take((size_t)a.x5_blocks * 2 * 8);
   const size_t o_sums = take(64 * 8);
   const size_t o_ctrl = take(sizeof(Ctrl));
