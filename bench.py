@@ -202,7 +202,7 @@ class ClockSampler:
 # pass must touch is counted once: eta_x reads eps (n_c scalars) and the phase
 # (1 B) per voxel; fwd_x reads the same and writes n_c half-spectrum
 # components; mid_y_fwd, fourier_z and mid_y_inv read and write n_c components;
-# inv_x reads n_c components, eps and the phase and writes eps.  Halo re-reads
+# inv_x reads n_c components, eps and the phase and writes eps; turn_x does that and writes n_c components.  Halo re-reads
 # are not counted.
 def kernel_bytes(kind, n, nc=6):
     prec = 8 if kind.endswith("f64") else 4
@@ -218,6 +218,8 @@ def kernel_bytes(kind, n, nc=6):
         return 2 * nc * half * cplx
     if k == "inv_x":
         return nc * half * cplx + N * (2 * nc * prec + 1)
+    if k == "turn_x":
+        return 2 * nc * half * cplx + N * (2 * nc * prec + 1)
     return None
 
 

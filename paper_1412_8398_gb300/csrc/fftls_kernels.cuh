@@ -129,6 +129,11 @@ struct IterArgs {
   int x5_lines, x5_blocks;  // inverse x1 pass
   int x5_vb;                // inverse x1 pass: 1 register loads of eps, 0 staged by bulk copies (FP32)
   int x_threads;
+  // x1 turn (fftls_turn.cuh): its twiddles (register variant), blocks (the separate x1 passes run on the
+  // same grid, so the partial sums of <sigma>, <eps> have one count), lines per tile or block, threads
+  const T2* twt;
+  int x_blocks, t_reg, t_lines, t_threads;  // t_reg: the register variant
+  size_t t_smem;
   int y_w, y_threads, z_w, z_threads;
   size_t x1_smem, x5_smem, y_smem, z_smem;
   int e_planes, e_blocks;  // real-space eta: x3-planes per block, blocks (tiles x slabs)
@@ -161,6 +166,15 @@ template <typename T> cudaError_t set_attrs_xgrp(size_t smax);
 template <typename T> cudaError_t set_attrs_ygrp(size_t smax);
 template <typename T> cudaError_t set_attrs_zgrp(size_t smax);
 
+// Lengths n1 of the x1 turn's register variant (fftls_turn.cuh).
+__host__ __device__ constexpr bool turn_reg_length(int n1) { return ct_length(n1); }
+// Entries of the turn's twiddle table: w_L^{j r} at [(r - 1) M + j], r = 1..7, j < M = L / 8, then w_M^{j t}
+// at [7 M + (t - 1) R2 + j], t = 1..R1-1, j < R2 (M = R1 R2, R1 = 4 for L = 128, else 8).
+__host__ __device__ constexpr int turn_r1(int L) { return L == 128 ? 4 : 8; }
+__host__ __device__ constexpr int turn_tw_count(int L) {
+  return turn_reg_length(L) ? 7 * (L / 8) + (turn_r1(L) - 1) * (L / 8 / turn_r1(L)) : 0;
+}
+
 // Launchers (fftls_kernels.cu).  All return cudaGetLastError().
 template <typename T> cudaError_t launch_fwd_x(const IterArgs<T>& a, cudaStream_t s);
 template <typename T> cudaError_t launch_eta_stencil(const IterArgs<T>& a, cudaStream_t s);
@@ -171,6 +185,11 @@ template <typename T> cudaError_t launch_fourier_z(const IterArgs<T>& a, cudaStr
 template <typename T> cudaError_t launch_reduce_eta(const IterArgs<T>& a, cudaStream_t s);
 template <typename T> cudaError_t launch_inv_x(const IterArgs<T>& a, cudaStream_t s);
 template <typename T> cudaError_t launch_reduce_delta(const IterArgs<T>& a, cudaStream_t s);
+// the x1 turn (fftls_kernels_t32.cu, _t64.cu), its dynamic shared-memory limit and need: `lines` per block of
+// the register variant, or per tile of the other (line: bytes of one)
+template <typename T> cudaError_t launch_turn(const IterArgs<T>& a, cudaStream_t s);
+template <typename T> cudaError_t set_attrs_turn(size_t smax);
+template <typename T> size_t turn_smem_reg(int n1, int npairs, int lines);
 template <typename T> cudaError_t set_kernel_attributes(const IterArgs<T>& a, size_t smax);
 // dynamic shared-memory limits of the x2 and x3 kernels (their own translation units)
 template <typename T> cudaError_t set_attrs_y(size_t smax);

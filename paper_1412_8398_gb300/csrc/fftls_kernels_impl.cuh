@@ -1911,6 +1911,7 @@ cudaError_t set_kernel_attributes(const IterArgs<T>& a, size_t smax) {
   if (e == cudaSuccess) e = set_attrs_y<T>(smax);
   if (e == cudaSuccess) e = set_attrs_z<T>(smax);
   if (e == cudaSuccess) e = set_attrs_grp<T>(smax);
+  if (e == cudaSuccess) e = set_attrs_turn<T>(smax);
   return e;
 }
 #undef FFTLS_ATTR

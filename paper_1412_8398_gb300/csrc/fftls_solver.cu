@@ -21,12 +21,12 @@ using namespace fftls;
 namespace {
 
 constexpr int kMaxL = 2048;
-constexpr int kNumKinds = 8;
+constexpr int kNumKinds = 9;
 const char* const kKindNames[2][kNumKinds] = {
     {"fwd_x_f32", "mid_y_fwd_f32", "fourier_z_f32", "reduce_eta_f32", "mid_y_inv_f32", "inv_x_f32",
-     "reduce_delta_f32", "eta_x_f32"},
+     "reduce_delta_f32", "eta_x_f32", "turn_x_f32"},
     {"fwd_x_f64", "mid_y_fwd_f64", "fourier_z_f64", "reduce_eta_f64", "mid_y_inv_f64", "inv_x_f64",
-     "reduce_delta_f64", "eta_x_f64"}};
+     "reduce_delta_f64", "eta_x_f64", "turn_x_f64"}};
 constexpr int kMaxOuter = 8;  // FP64 residual evaluations of the refinement ladder
 constexpr int kMaxWorkers = 64, kDefaultWorkers = 8;  // concurrent solves of fftls_solve_batched
 // grouped launches of fftls_solve_batched: samples per group, and the device memory a
@@ -379,7 +379,28 @@ size_t table_offset_kt(const Setup& S, int ax) {
   return table_offset_tw(S, ax) + 2 * (size_t)fftls::tw_count(S.pl[ax].L, tw_layout(ax));
 }
 size_t table_offset_rd(const Setup& S, int ax) { return table_offset_kt(S, ax) + 6 * (size_t)S.pl[ax].L; }
-size_t table_count(const Setup& S) { return table_offset_tw(S, 3); }
+size_t table_offset_turn(const Setup& S) { return table_offset_tw(S, 3); }
+size_t table_count(const Setup& S) { return table_offset_turn(S) + 2 * (size_t)fftls::turn_tw_count(S.g.n1); }
+
+// Twiddles of the x1 turn's register variant (layout: turn_tw_count).
+void turn_twiddles(int L, double* tw) {
+  const int M = L / 8, R1 = fftls::turn_r1(L), R2 = M / R1;
+  auto put = [&](int at, int t) {  // e^{-2 pi i t / L}, exact at multiples of pi / 2
+    const double ang = -2.0 * M_PI * (double)t / (double)L;
+    double cs = cos(ang), sn = sin(ang);
+    if ((4 * t) % L == 0) {
+      const double cq[4] = {1, 0, -1, 0}, sq[4] = {0, -1, 0, 1};
+      cs = cq[(4 * t / L) % 4];
+      sn = sq[(4 * t / L) % 4];
+    }
+    tw[2 * at] = cs;
+    tw[2 * at + 1] = sn;
+  };
+  for (int r = 1; r < 8; ++r)
+    for (int j = 0; j < M; ++j) put((r - 1) * M + j, j * r);
+  for (int t = 1; t < R1; ++t)
+    for (int j = 0; j < R2; ++j) put(7 * M + (t - 1) * R2 + j, 8 * j * t);
+}
 
 // Fill the table block (tab) and the per-axis permutations (perms: storage position ->
 // frequency, then frequency -> position, per axis).  No heap allocation (the
@@ -394,6 +415,7 @@ void fill_tables(const Setup& S, double* tab, int* perms) {
                 &tab[table_offset_kt(S, ax)], &tab[table_offset_rd(S, ax)]);
     po += 2 * (size_t)L;
   }
+  if (fftls::turn_reg_length(S.g.n1)) turn_twiddles(S.g.n1, &tab[table_offset_turn(S)]);
 }
 
 void build_tables(const Setup& S, std::vector<double>& tab, std::vector<int>& perms) {
@@ -422,6 +444,12 @@ PlanGeom plan_geom(const Setup& S, size_t cb, bool real_eta) {
   G.nlines = (long long)S.g.n2 * S.g.n3;
   G.tiles = (long long)((S.g.n1 + kEtaTileX - 1) / kEtaTileX) * ((S.g.n2 + kEtaTileY - 1) / kEtaTileY);
   return G;
+}
+
+// Whether the x1 turn runs its register variant: one of its lengths, and at least 64 threads (n1 / 8 per
+// line) for every SM (see fftls_turn.cuh).
+bool turn_reg(const Setup& S) {
+  return fftls::turn_reg_length(S.g.n1) && (long long)S.g.n2 * S.g.n3 * (S.g.n1 / 8) >= 64LL * S.num_sms;
 }
 
 size_t strided_smem(int L, int w, int nc, size_t cb) {
@@ -481,8 +509,26 @@ bool apply_plan(const Setup& S, IterArgs<T>& a, bool real_eta, const TilePlan& P
     if (a.x5_smem > G.lim) return false;
   }
   a.x_threads = 256;
-  a.x1_blocks = (int)std::min<long long>((G.nlines + G1 - 1) / G1, (long long)S.num_sms * 8);
-  a.x5_blocks = (int)std::min<long long>((G.nlines + G5 - 1) / G5, (long long)S.num_sms * 8);
+  // x1 turn: the register variant takes blocks of 128 threads, fewer while the lines would leave SMs
+  // without a block; the other tiles of the inverse pass's lines, as far as they fit with rows wide enough
+  // to carry sigma too wherever eta is taken in Fourier space (the accelerated scheme, and the correction
+  // phases of both schemes)
+  a.t_reg = turn_reg(S) ? 1 : 0;
+  if (a.t_reg) {
+    const int M = g.n1 / 8;
+    a.t_threads = 128;
+    while (a.t_threads > std::max(32, M) && G.nlines * M / a.t_threads < S.num_sms) a.t_threads /= 2;
+    a.t_lines = a.t_threads / M;
+    a.t_smem = turn_smem_reg<T>(g.n1, (S.nc + 1) / 2, a.t_lines);
+  } else {
+    const size_t line = real_eta ? G.line5 : (size_t)padded_rows(g.n1) * odd_up(S.nc) * sizeof(T2);
+    a.t_threads = 256;
+    a.t_lines = (int)std::min<size_t>(G5, (G.lim - G.twx) / line);
+    if (a.t_lines < 1) return false;
+    a.t_smem = G.twx + a.t_lines * line;
+  }
+  a.x_blocks = (int)std::min<long long>((G.nlines + a.t_lines - 1) / a.t_lines, (long long)S.num_sms * 8);
+  a.x1_blocks = a.x5_blocks = a.x_blocks;
   // 2D: the Fourier pass works on x2 tiles (the x2 pass's width) and the x2 pass does not run
   a.y_w = P.y_w;
   a.z_w = S.dim == 3 ? P.z_w : P.y_w;
@@ -522,7 +568,7 @@ struct Runner {
   Runner(fftls_ctx* c_, const Setup& S_) : c(c_), S(S_), hctl(c_->h_ctrl) { memset(&a, 0, sizeof(a)); }
 
   bool has_mid_y() const { return S.dim == 3 && S.g.n2 > 1; }
-  int kernels_per_iter() const { return 4 + (has_mid_y() ? 2 : 0) + (a.want_delta ? 1 : 0) + (a.eta_real ? 1 : 0); }
+  int kernels_per_iter() const { return 3 + (has_mid_y() ? 2 : 0) + (a.want_delta ? 1 : 0) + (a.eta_real ? 1 : 0); }
 
   fftls_status launch(int kind, cudaError_t (*fn)(Runner*, cudaStream_t), bool prof) {
     const int pi = Prec<T>::idx;
@@ -543,6 +589,8 @@ struct Runner {
     return FFTLS_OK;
   }
 
+  // One iteration of separate x1 passes: forward, the strided passes and the stop decision, inverse with
+  // the update (the FP64 defect of the ladder, and the tau-form step of a warm-started direct solve).
   fftls_status iteration(bool dual, int update, bool prof) {
     a.dual = (dual && !a.eta_real) ? 1 : 0;
     a.tauform = (a.dual || a.eta_real) ? 1 : 0;
@@ -556,6 +604,23 @@ struct Runner {
     if ((st = launch(3, [](Runner* r, cudaStream_t s) { return launch_reduce_eta<T>(r->a, s); }, prof))) return st;
     if ((st = launch(4, [](Runner* r, cudaStream_t s) { return launch_mid_y<T>(r->a, true, s); }, prof))) return st;
     if ((st = launch(5, [](Runner* r, cudaStream_t s) { return launch_inv_x<T>(r->a, s); }, prof))) return st;
+    if (a.want_delta)
+      if ((st = launch(6, [](Runner* r, cudaStream_t s) { return launch_reduce_delta<T>(r->a, s); }, prof)))
+        return st;
+    return FFTLS_OK;
+  }
+
+  // One iteration in steady state: the spectrum of the iterate's polarisation is there (from the forward
+  // pass before the first one, then from each x1 turn); the turn leaves the next iterate's.
+  fftls_status turn_iteration(bool prof) {
+    fftls_status st;
+    if (a.eta_real)
+      if ((st = launch(7, [](Runner* r, cudaStream_t s) { return launch_eta_stencil<T>(r->a, s); }, prof))) return st;
+    if ((st = launch(1, [](Runner* r, cudaStream_t s) { return launch_mid_y<T>(r->a, false, s); }, prof))) return st;
+    if ((st = launch(2, [](Runner* r, cudaStream_t s) { return launch_fourier_z<T>(r->a, s); }, prof))) return st;
+    if ((st = launch(3, [](Runner* r, cudaStream_t s) { return launch_reduce_eta<T>(r->a, s); }, prof))) return st;
+    if ((st = launch(4, [](Runner* r, cudaStream_t s) { return launch_mid_y<T>(r->a, true, s); }, prof))) return st;
+    if ((st = launch(8, [](Runner* r, cudaStream_t s) { return launch_turn<T>(r->a, s); }, prof))) return st;
     if (a.want_delta)
       if ((st = launch(6, [](Runner* r, cudaStream_t s) { return launch_reduce_delta<T>(r->a, s); }, prof)))
         return st;
@@ -634,13 +699,14 @@ struct Runner {
       if ((st = read_ctrl())) return st;
       if (!running()) return FFTLS_OK;
     }
+    a.dual = (dual && !a.eta_real) ? 1 : 0;
+    a.tauform = (a.dual || a.eta_real) ? 1 : 0;
+    a.update = update;
+    if ((st = launch(0, [](Runner* r, cudaStream_t s) { return launch_fwd_x<T>(r->a, s); }, S.profile))) return st;
     const long long N = S.g.N * ns;
     const int chunk = (int)std::max<long long>(1, std::min<long long>(32, 40000000LL / std::max<long long>(N, 1)));
     cudaGraphExec_t exec = nullptr;
     if (S.graphs && !S.profile) {
-      a.dual = (dual && !a.eta_real) ? 1 : 0;
-      a.tauform = (a.dual || a.eta_real) ? 1 : 0;
-      a.update = update;
       GraphCache& gc = c->graphs[Prec<T>::idx];
       std::vector<unsigned char> key(sizeof(a) + sizeof(int));
       memcpy(key.data(), &a, sizeof(a));
@@ -653,7 +719,7 @@ struct Runner {
         CUDA_TRY(c, cudaStreamBeginCapture(S.s, cudaStreamCaptureModeThreadLocal));
         fftls_status cs = FFTLS_OK;
         capturing = true;
-        for (int i = 0; i < chunk && cs == FFTLS_OK; ++i) cs = iteration(dual, update, false);
+        for (int i = 0; i < chunk && cs == FFTLS_OK; ++i) cs = turn_iteration(false);
         capturing = false;
         cudaError_t ce = cudaStreamEndCapture(S.s, &graph);
         if (cs) return cs;
@@ -672,7 +738,7 @@ struct Runner {
         c->launches += (long long)chunk * kernels_per_iter();
       } else {
         for (int i = 0; i < chunk; ++i)
-          if ((st = iteration(dual, update, S.profile))) return st;
+          if ((st = turn_iteration(S.profile))) return st;
         if ((st = collect_profile())) return st;
       }
       if ((st = read_ctrl())) return st;
@@ -799,11 +865,16 @@ fftls_status tune_plan(fftls_ctx* c, const Setup& S, IterArgs<T>& a, bool real_e
     search_wt(&TilePlan::z_w, &TilePlan::z_thr, fourier);
   }
   a.eps = (T*)c->specB.p;  // scratch target of the inverse pass's update
-  // inverse x1 pass: lines per batch and (FP32) eps loaded by the threads or staged by bulk copies, jointly
+  // x1 turn on tiles: lines per tile (it writes its update into the scratch
+  // iterate); the register variant has nothing to choose, and there the inverse x1 pass is timed: lines per
+  // batch and (FP32) eps loaded by the threads or staged by bulk copies, jointly
+  const bool turn_tiles = !turn_reg(S);
   {
     float best = INFINITY;
     int bl = P.x5_lines, bv = P.x5_vb;
-    const std::vector<int> vbs = sizeof(T) == 8 ? std::vector<int>{1} : std::vector<int>{1, 0};
+    const std::vector<int> vbs = sizeof(T) == 8 || turn_tiles ? std::vector<int>{1} : std::vector<int>{1, 0};
+    const LaunchFn pass = turn_tiles ? (LaunchFn)[](const IterArgs<T>& x, cudaStream_t st) { return launch_turn<T>(x, st); }
+                                     : (LaunchFn)[](const IterArgs<T>& x, cudaStream_t st) { return launch_inv_x<T>(x, st); };
     for (int lines : {1, 2, 4, 8})
       for (int vb : vbs) {
         if (err != cudaSuccess) break;
@@ -812,7 +883,7 @@ fftls_status tune_plan(fftls_ctx* c, const Setup& S, IterArgs<T>& a, bool real_e
         Q.x5_vb = vb;
         if (!apply_plan<T>(S, a, real_eta, Q)) continue;
         float ms = 0.f;
-        err = timed([](const IterArgs<T>& x, cudaStream_t st) { return launch_inv_x<T>(x, st); }, &ms);
+        err = timed(pass, &ms);
         c->launches += 1 + kReps;
         if (ms < best) {
           best = ms;
@@ -879,6 +950,7 @@ fftls_status prepare(fftls_ctx* c, const Setup& S, const fftls_problem* p, const
     a.pos[ax] = d_perms + po + S.pl[ax].L;
     po += 2 * (size_t)S.pl[ax].L;
   }
+  a.twt = (const T2*)((const T*)tb.p + table_offset_turn(S));
   a.eps = eps;
   a.phase = S.d_phase;
   a.specA = (T2*)c->specA.p;
@@ -1697,7 +1769,7 @@ void* g_noalloc_base[kNoAllocMaxDevices];  // device address of g_noalloc_scratc
 // so the arrays are free again when the lock is released)
 std::mutex g_na_lock;
 double g_na_coef[256 * kCoef];
-double g_na_tab[3 * (2 * (kMaxL + 2) + 8 * kMaxL)];
+double g_na_tab[3 * (2 * (kMaxL + 2) + 8 * kMaxL) + 2 * 1024];
 int g_na_perm[6 * kMaxL];
 
 size_t na_align(size_t x) { return (x + 255) & ~(size_t)255; }
