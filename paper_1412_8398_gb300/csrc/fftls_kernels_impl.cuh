@@ -134,6 +134,21 @@ __device__ __forceinline__ T2* load_twiddles(const T2* __restrict__ tw, int L, i
   return tws;
 }
 
+// The same for the strided passes, which may run beside the reduction that writes the solve's state: the
+// block decides as one (any thread that saw the solve going on keeps all of them) whether it works, at the
+// barrier that completes the table.  A state read by each thread for itself could differ within a block
+// while it changes, and half of the block would leave before the tile's copies and barriers.
+template <typename T2>
+__device__ __forceinline__ bool strided_begin(const Ctrl* ctl, const T2* __restrict__ tw, int L, T2** tws, T2** tile) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int st = ctl->state;
+  *tws = reinterpret_cast<T2*>(smem_raw);
+  const int n = tw_count(L, kTwStrided);
+  for (int t = threadIdx.x; t < n; t += blockDim.x) (*tws)[t] = tw[t];
+  *tile = *tws + n;
+  return __syncthreads_or(st == kRunning || st == kLast);
+}
+
 __host__ __device__ constexpr int odd_stride(int n) { return (n & 1) ? n : n + 1; }
 
 // 16-byte asynchronous copy global -> shared (bypasses registers and L1), so a
@@ -673,7 +688,7 @@ __device__ __forceinline__ int wrap_index(int i, int n) {
 
 template <typename T, bool CEN>
 __device__ __forceinline__ void k_eta_stencil_body(const IterArgs<T>& a, const AxisPlan* pl) {
-  if (a.ctrl->state != kRunning) return;
+  if (!__syncthreads_or(a.ctrl->state == kRunning)) return;  // block-uniform: a strided pass beside it may stop the solve
   const Geom g = a.g;
   const int n1 = g.n1, n2 = g.n2, n3 = g.n3;
   const long long N = g.N;
@@ -817,12 +832,10 @@ template <typename T, int NC, int W>
 __device__ __forceinline__ void k_mid_y_body(const IterArgs<T>& a, const AxisPlan* pl, int inv, int kind) {
   typedef typename Cplx<T>::type T2;
   constexpr int NT = strided_threads(W);
-  const int st = a.ctrl->state;
-  if (inv ? (st != kRunning && st != kLast) : (st != kRunning)) return;
   const Geom g = a.g;
   const int n2 = g.n2;
-  T2* tile;
-  const T2* tws = load_twiddles(a.tw[1], n2, kTwStrided, &tile);
+  T2 *tws, *tile;
+  if (!strided_begin(a.ctrl, a.tw[1], n2, &tws, &tile)) return;
   const int x0 = blockIdx.x * W;
   const int nx = min(W, g.H - x0);
   constexpr int C = W * NC;
@@ -1168,11 +1181,10 @@ __device__ __forceinline__ void k_fourier_z_body(const IterArgs<T>& a, const Axi
   // pass with n3 = 1 between two x2 passes, a block had one row of at most 16 modes for its 256
   // threads: 512^2 FP64, G^R accelerated, 542 -> 245 us per iteration; 128^2, direct, 63 -> 44 us.)
   constexpr int AX = DIM - 1;
-  if (a.ctrl->state != kRunning) return;
   const Geom g = a.g;
   const int nl = DIM == 3 ? g.n3 : g.n2;
-  T2* tile;
-  const T2* tws = load_twiddles(a.tw[AX], nl, kTwStrided, &tile);
+  T2 *tws, *tile;
+  if (!strided_begin(a.ctrl, a.tw[AX], nl, &tws, &tile)) return;
   const int x0 = blockIdx.x * W;
   const int py = DIM == 3 ? blockIdx.y : 0;
   const bool do_green = kind == 0;
@@ -1289,7 +1301,7 @@ __device__ __forceinline__ void k_reduce_eta_body(const IterArgs<T>& a, const Ax
   constexpr int NC = Comp<DIM>::NC;
   Ctrl* ctl = a.ctrl;
   const int st = ctl->state;
-  if (st != kRunning || ctl->it >= ctl->max_it) {
+  if (!__syncthreads_or(st == kRunning && ctl->it < ctl->max_it)) {  // block-uniform, as strided_begin
     if (threadIdx.x == 0 && (st == kLast || st == kRunning)) ctl->state = kStopped;
     return;
   }
