@@ -1,5 +1,6 @@
 // Kernel interfaces of the FFT Lippmann-Schwinger iteration (internal header).
 #pragma once
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -79,6 +80,8 @@ struct KTab {
 // with a_kappa = kappa0 / (kappa + kappa0), a_mu = mu0 / (mu + mu0).
 constexpr int kCoef = 8;
 
+constexpr int kSmpPar = 10;  // doubles per sample in IterArgs::smp_par
+
 template <typename T>
 struct IterArgs {
   typedef typename Cplx<T>::type T2;
@@ -101,12 +104,15 @@ struct IterArgs {
   const T2* tw[3];   // per axis: e^{-2 pi i t / L}
   const KTab<T>* kt[3];
   const T2* rd[3];     // per axis, by storage position: {a, b} with kr_i = a_i prod_{m != i} b_m
-                       // (G^R: a = 2 sin(q/2), b = cos(q/2); G^C: a = sin q, b = 1; G: a = q, b = 1)
+                       // (G^R: a = 2 sin(q/2), b = cos(q/2); G^C: a = sin q, b = 1; G: a = q, b = 1);
+                       // G^W: {cos q - 1, sin q}, the axis's k itself
+  const float4* tws[3];  // x2, x3: twiddles of the FP32 register passes {w.x, w.x, w.y, w.y} (fftls_strided.cuh)
   const int* perm[3];  // per axis: storage position -> frequency index
   const int* pos[3];   // per axis: frequency index -> storage position
   AxisPlan pl[3];
   double lam0, mu0;
   double eps_bar[6];
+  T green_cf, green_c0, inv_n;  // -1 / (N mu0), (lambda0 + mu0) / (lambda0 + 2 mu0), 1 / N
   Ctrl* ctrl;
   double* part_mean;   // [x1_blocks][2 nc]: sums of sigma and eps per block
   double* part_eta;    // [z blocks or eta blocks]: sums of |k*.sigma_hat|^2 per block
@@ -118,7 +124,7 @@ struct IterArgs {
                        // eta_real [3][N] floats: its real-space divergence
   // grouped launches (fftls_solve_batched): nsmp samples of one 3D geometry share a
   // launch; sample s finds its fields at these element offsets times s (null fields:
-  // offset 0) and its lambda0, mu0, eps_bar[6] at smp_par[8 s ..] (device memory).
+  // offset 0) and its lambda0, mu0, eps_bar[6], green_cf, green_c0 at smp_par[kSmpPar s ..] (device memory).
   // Single solves have nsmp = 1 and use the values above.
   int nsmp;
   long long st_field, st_phase, st_spec, st_coef, st_pmean, st_peta, st_pdelta, st_hist, st_d64;
@@ -136,6 +142,7 @@ struct IterArgs {
   size_t t_smem;
   int y_w, y_threads, z_w, z_threads;
   size_t x1_smem, x5_smem, y_smem, z_smem;
+  CUtensorMap tm[3];       // FP32 register passes: x2 boxes of specA, of specB, x3 boxes of specA (set per launch)
   int e_planes, e_blocks;  // real-space eta: x3-planes per block, blocks (tiles x slabs)
   size_t e_smem;
 };
@@ -190,6 +197,16 @@ template <typename T> cudaError_t launch_reduce_delta(const IterArgs<T>& a, cuda
 template <typename T> cudaError_t launch_turn(const IterArgs<T>& a, cudaStream_t s);
 template <typename T> cudaError_t set_attrs_turn(size_t smax);
 template <typename T> size_t turn_smem_reg(int n1, int npairs, int lines);
+// Entries of a register pass's twiddle table: w_M^{j r} of stage s at the stage's offset + (r - 1) MR + j
+__host__ __device__ constexpr int strided_reg_tw(int L, int s) {
+  return s == 0 ? 0 : strided_reg_tw(L, s - 1) + (ct_radix(L, s - 1) - 1) * (ct_msize(L, s - 1) / ct_radix(L, s - 1));
+}
+// FP32 register passes along x2 and x3 (fftls_strided.cuh, fftls_kernels_yr32.cu, _zr32.cu) and their lengths
+__host__ __device__ constexpr bool strided_reg_length(int L) { return ct_length(L); }
+cudaError_t launch_y_reg(const IterArgs<float>& a, bool inv, cudaStream_t s);
+cudaError_t launch_z_reg(const IterArgs<float>& a, cudaStream_t s);
+cudaError_t set_attrs_y_reg();
+cudaError_t set_attrs_z_reg();
 template <typename T> cudaError_t set_kernel_attributes(const IterArgs<T>& a, size_t smax);
 // dynamic shared-memory limits of the x2 and x3 kernels (their own translation units)
 template <typename T> cudaError_t set_attrs_y(size_t smax);

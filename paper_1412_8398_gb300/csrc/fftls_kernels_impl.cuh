@@ -47,7 +47,7 @@ __device__ __forceinline__ void at_sample(IterArgs<T>& a, int s) {
   a.ms_hist += s * a.st_hist * 6;
   a.rfield += s * a.st_field;
   a.d64 += s * a.st_d64;
-  const double* p = a.smp_par + 8 * s;
+  const double* p = a.smp_par + kSmpPar * s;
   a.lam0 = p[0];
   a.mu0 = p[1];
 #pragma unroll
@@ -1810,8 +1810,16 @@ cudaError_t launch_reduce_delta_t(const IterArgs<T>& a, cudaStream_t s) {
 #define FFTLS_PICK(fn, ...) (a.nsmp > 1 ? fn##_grp<T>(__VA_ARGS__) : fn##_t<T, false>(__VA_ARGS__))
 template <typename T> cudaError_t launch_fwd_x(const IterArgs<T>& a, cudaStream_t s) { return FFTLS_PICK(launch_fwd_x, a, s); }
 template <typename T> cudaError_t launch_eta_stencil(const IterArgs<T>& a, cudaStream_t s) { return FFTLS_PICK(launch_eta_stencil, a, s); }
-template <typename T> cudaError_t launch_mid_y(const IterArgs<T>& a, bool inv, cudaStream_t s) { return FFTLS_PICK(launch_mid_y, a, inv, s); }
-template <typename T> cudaError_t launch_fourier_z(const IterArgs<T>& a, cudaStream_t s) { return FFTLS_PICK(launch_fourier_z, a, s); }
+template <typename T> cudaError_t launch_mid_y(const IterArgs<T>& a, bool inv, cudaStream_t s) {
+  if constexpr (sizeof(T) == 4)
+    if (a.dim == 3 && strided_reg_length(a.g.n2)) return launch_y_reg(a, inv, s);
+  return FFTLS_PICK(launch_mid_y, a, inv, s);
+}
+template <typename T> cudaError_t launch_fourier_z(const IterArgs<T>& a, cudaStream_t s) {
+  if constexpr (sizeof(T) == 4)
+    if (a.dim == 3 && a.eta_real && strided_reg_length(a.g.n3)) return launch_z_reg(a, s);
+  return FFTLS_PICK(launch_fourier_z, a, s);
+}
 template <typename T> cudaError_t launch_reduce_eta(const IterArgs<T>& a, cudaStream_t s) { return FFTLS_PICK(launch_reduce_eta, a, s); }
 template <typename T> cudaError_t launch_inv_x(const IterArgs<T>& a, cudaStream_t s) { return FFTLS_PICK(launch_inv_x, a, s); }
 template <typename T> cudaError_t launch_reduce_delta(const IterArgs<T>& a, cudaStream_t s) { return FFTLS_PICK(launch_reduce_delta, a, s); }
@@ -1924,6 +1932,10 @@ cudaError_t set_kernel_attributes(const IterArgs<T>& a, size_t smax) {
   if (e == cudaSuccess) e = set_attrs_z<T>(smax);
   if (e == cudaSuccess) e = set_attrs_grp<T>(smax);
   if (e == cudaSuccess) e = set_attrs_turn<T>(smax);
+  if (sizeof(T) == 4) {
+    if (e == cudaSuccess) e = set_attrs_y_reg();
+    if (e == cudaSuccess) e = set_attrs_z_reg();
+  }
   return e;
 }
 #undef FFTLS_ATTR

@@ -114,7 +114,7 @@ void plan_permutation(const AxisPlan& p, int* perm, int* pos) {
 // wave-vector table {q, sin q, cos q - 1, sin q/2, cos q/2, nyquist} by frequency
 // index, and the real-direction factors {a, b} of operator `green` by storage
 // position p (frequency perm[p]; perm = NULL: natural order): kr_i = a_i prod_{m != i} b_m, with
-// G^R: a = 2 sin(q/2), b = cos(q/2);  G^C: a = sin q, b = 1;  G: a = q, b = 1.
+// G^R: a = 2 sin(q/2), b = cos(q/2);  G^C: a = sin q, b = 1;  G: a = q, b = 1;  G^W: k = a + i b.
 void axis_tables(int L, int layout, int green, const int* perm, double* tw, double* kt, double* rd) {
   static_assert(fftls::tw_count(512, fftls::kTwStrided) <= kMaxL + 2, "stage twiddle rows fit the plain table's bound");
   double plain[2 * kMaxL];
@@ -171,6 +171,7 @@ void axis_tables(int L, int layout, int green, const int* perm, double* tw, doub
     if (green == FFTLS_GREEN_R) { av = 2.0 * e[3]; bv = e[4]; }
     else if (green == FFTLS_GREEN_C) av = e[1];
     else if (green == FFTLS_GREEN_MS) av = e[0];
+    else { av = e[2]; bv = e[1]; }  // G^W: k itself
     rd[2 * (size_t)p] = av;
     rd[2 * (size_t)p + 1] = bv;
   }
@@ -382,7 +383,34 @@ size_t table_offset_kt(const Setup& S, int ax) {
 }
 size_t table_offset_rd(const Setup& S, int ax) { return table_offset_kt(S, ax) + 6 * (size_t)S.pl[ax].L; }
 size_t table_offset_turn(const Setup& S) { return table_offset_tw(S, 3); }
-size_t table_count(const Setup& S) { return table_offset_turn(S) + 2 * (size_t)fftls::turn_tw_count(S.g.n1); }
+// ... and of the FP32 register passes along x2 and x3 (four values an entry)
+size_t strided_reg_count(int L) { return fftls::strided_reg_length(L) ? (size_t)fftls::strided_reg_tw(L, fftls::ct_nst(L)) : 0; }
+size_t table_offset_reg(const Setup& S, int ax) {
+  size_t off = table_offset_turn(S) + 2 * (size_t)fftls::turn_tw_count(S.g.n1);
+  off = (off + 3) & ~(size_t)3;
+  return ax == 2 ? off + 4 * strided_reg_count(S.g.n2) : off;
+}
+size_t table_count(const Setup& S) { return table_offset_reg(S, 2) + 4 * strided_reg_count(S.g.n3); }
+
+void reg_twiddles(int L, double* tw) {
+  for (int s = 0; s < fftls::ct_nst(L); ++s) {
+    const int R = fftls::ct_radix(L, s), M = fftls::ct_msize(L, s), MR = M / R;
+    for (int r = 1; r < R; ++r)
+      for (int j = 0; j < MR; ++j) {
+        double* e = tw + 4 * (size_t)(fftls::strided_reg_tw(L, s) + (r - 1) * MR + j);
+        const int t = (r * j * (L / M)) % L;  // e^{-2 pi i t / L}, exact at multiples of pi / 2
+        const double ang = -2.0 * M_PI * (double)t / (double)L;
+        double cs = cos(ang), sn = sin(ang);
+        if ((4 * t) % L == 0) {
+          const double cq[4] = {1, 0, -1, 0}, sq[4] = {0, -1, 0, 1};
+          cs = cq[(4 * t / L) % 4];
+          sn = sq[(4 * t / L) % 4];
+        }
+        e[0] = e[1] = cs;
+        e[2] = e[3] = sn;
+      }
+  }
+}
 
 // Twiddles of the x1 turn's register variant (layout: turn_tw_count).
 void turn_twiddles(int L, double* tw) {
@@ -406,8 +434,9 @@ void turn_twiddles(int L, double* tw) {
 
 // Fill the table block (tab) and the per-axis permutations (perms: storage position ->
 // frequency, then frequency -> position, per axis).  No heap allocation (the
-// allocation-free entry point stages its tables through here).
-void fill_tables(const Setup& S, double* tab, int* perms) {
+// allocation-free entry point stages its tables through here, without those of the register
+// passes: reg false, table_offset_turn values).
+void fill_tables(const Setup& S, double* tab, int* perms, bool reg = true) {
   size_t po = 0;
   for (int ax = 0; ax < 3; ++ax) {
     const int L = S.pl[ax].L;
@@ -417,7 +446,10 @@ void fill_tables(const Setup& S, double* tab, int* perms) {
                 &tab[table_offset_kt(S, ax)], &tab[table_offset_rd(S, ax)]);
     po += 2 * (size_t)L;
   }
+  if (!reg) return;
   if (fftls::turn_reg_length(S.g.n1)) turn_twiddles(S.g.n1, &tab[table_offset_turn(S)]);
+  if (fftls::strided_reg_length(S.g.n2)) reg_twiddles(S.g.n2, &tab[table_offset_reg(S, 1)]);
+  if (fftls::strided_reg_length(S.g.n3)) reg_twiddles(S.g.n3, &tab[table_offset_reg(S, 2)]);
 }
 
 void build_tables(const Setup& S, std::vector<double>& tab, std::vector<int>& perms) {
@@ -933,6 +965,11 @@ fftls_status tune_plan(fftls_ctx* c, const Setup& S, IterArgs<T>& a, bool real_e
   return FFTLS_OK;
 }
 
+// -1 / (N mu0) and (lambda0 + mu0) / (lambda0 + 2 mu0) of the real-direction Gamma'
+double green_factor(const Setup& S, int which) {
+  return which ? (S.lam0 + S.mu0) / (S.lam0 + 2.0 * S.mu0) : -1.0 / ((double)S.g.N * S.mu0);
+}
+
 template <typename T>
 fftls_status prepare(fftls_ctx* c, const Setup& S, const fftls_problem* p, const fftls_options* o, Runner<T>& R,
                      T* eps, const std::vector<double>& tab, const int* d_perms) {
@@ -976,6 +1013,11 @@ fftls_status prepare(fftls_ctx* c, const Setup& S, const fftls_problem* p, const
     po += 2 * (size_t)S.pl[ax].L;
   }
   a.twt = (const T2*)((const T*)tb.p + table_offset_turn(S));
+  if (sizeof(T) == 4)
+    for (int ax = 1; ax < 3; ++ax) a.tws[ax] = (const float4*)((const T*)tb.p + table_offset_reg(S, ax));
+  a.green_cf = (T)green_factor(S, 0);
+  a.green_c0 = (T)green_factor(S, 1);
+  a.inv_n = (T)(1.0 / (double)S.g.N);
   a.eps = eps;
   a.phase = S.d_phase;
   a.specA = (T2*)c->specA.p;
@@ -1326,12 +1368,15 @@ static fftls_status solve_core(fftls_ctx* c, const fftls_problem* const* P, int 
     Rn.ns = ns;
     Rn.hctl = hctl;
     if (ns == 1) return FFTLS_OK;
-    std::vector<double> cf((size_t)ns * 256 * kCoef), par((size_t)ns * 8);
+    std::vector<double> cf((size_t)ns * 256 * kCoef), par((size_t)ns * kSmpPar);
     for (int i = 0; i < ns; ++i) {
       coef_table(Ss[i], P[i], &cf[(size_t)i * 256 * kCoef]);
-      par[8 * (size_t)i] = Ss[i].lam0;
-      par[8 * (size_t)i + 1] = Ss[i].mu0;
-      for (int k = 0; k < 6; ++k) par[8 * (size_t)i + 2 + k] = Ss[i].eps_bar[k];
+      double* pi = &par[kSmpPar * (size_t)i];
+      pi[0] = Ss[i].lam0;
+      pi[1] = Ss[i].mu0;
+      for (int k = 0; k < 6; ++k) pi[2 + k] = Ss[i].eps_bar[k];
+      pi[8] = green_factor(Ss[i], 0);
+      pi[9] = green_factor(Ss[i], 1);
     }
     std::vector<T> cfT(cf.begin(), cf.end());
     DevBuf& cb = Prec<T>::idx ? c->coef64 : c->coef32;
@@ -1800,7 +1845,7 @@ void* g_noalloc_base[kNoAllocMaxDevices];  // device address of g_noalloc_scratc
 // so the arrays are free again when the lock is released)
 std::mutex g_na_lock;
 double g_na_coef[256 * kCoef];
-double g_na_tab[3 * (2 * (kMaxL + 2) + 8 * kMaxL) + 2 * 1024];
+double g_na_tab[3 * (2 * (kMaxL + 2) + 8 * kMaxL)];
 int g_na_perm[6 * kMaxL];
 
 size_t na_align(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -1842,6 +1887,10 @@ extern "C" fftls_status fftls_solve_noalloc(const fftls_problem* p, const fftls_
   IterArgs<double> a;
   memset(&a, 0, sizeof(a));
   if (!apply_plan<double>(S, a, false, default_plan(S, sizeof(double2), false))) return FFTLS_E_UNSUPPORTED_SIZE;
+  // its separate x1 passes take a block per batch of their own lines
+  const long long nlines = (long long)S.g.n2 * S.g.n3;
+  a.x1_blocks = (int)std::min<long long>((nlines + a.x1_lines - 1) / a.x1_lines, (long long)S.num_sms * 8);
+  a.x5_blocks = (int)std::min<long long>((nlines + a.x5_lines - 1) / a.x5_lines, (long long)S.num_sms * 8);
   // scratch layout
   const int ntz = (S.g.H + a.z_w - 1) / a.z_w;
   const int sblocks = (int)std::min<long long>((N + 255) / 256, (long long)S.num_sms * 8);
@@ -1857,7 +1906,7 @@ extern "C" fftls_status fftls_solve_noalloc(const fftls_problem* p, const fftls_
   const size_t o_eh = take((size_t)o->max_iter * 8);
   const size_t o_mh = take((size_t)o->max_iter * nc * 8);
   const size_t o_coef = take(256 * kCoef * 8);
-  const size_t ntab = table_count(S);
+  const size_t ntab = table_offset_turn(S);
   const size_t o_tab = take(ntab * 8);
   const size_t nperm = 2 * (size_t)(S.g.n1 + S.g.n2 + S.g.n3);
   const size_t o_perm = take(nperm * sizeof(int));
@@ -1869,7 +1918,7 @@ extern "C" fftls_status fftls_solve_noalloc(const fftls_problem* p, const fftls_
     std::lock_guard<std::mutex> lk(g_na_lock);
     coef_table(S, p, g_na_coef);
     NA_TRY(cudaMemcpyAsync(base + o_coef, g_na_coef, sizeof(g_na_coef), cudaMemcpyHostToDevice, S.s));
-    fill_tables(S, g_na_tab, g_na_perm);
+    fill_tables(S, g_na_tab, g_na_perm, false);
     NA_TRY(cudaMemcpyAsync(base + o_tab, g_na_tab, ntab * 8, cudaMemcpyHostToDevice, S.s));
     NA_TRY(cudaMemcpyAsync(base + o_perm, g_na_perm, nperm * sizeof(int), cudaMemcpyHostToDevice, S.s));
   }
