@@ -23,16 +23,40 @@
 namespace fftls {
 
 constexpr int kMaxStages = 12;
-constexpr int kMaxRadix = 8;
+
+// Division by a runtime divisor 1 <= d < 2^31 through a multiply-high and a
+// shift (Granlund and Montgomery 1994), exact for 0 <= n < 2^31.
+struct FastDiv {
+  unsigned int m, s;
+  int d;
+};
+
+__host__ __device__ inline FastDiv make_fastdiv(int d) {
+  unsigned int l = 0;
+  while ((1u << l) < (unsigned int)d) ++l;
+  const unsigned long long m = ((1ull << 32) * ((1ull << l) - (unsigned long long)d)) / (unsigned long long)d + 1ull;
+  FastDiv f;
+  f.m = (unsigned int)m;
+  f.s = l;
+  f.d = d;
+  return f;
+}
+
+__device__ __forceinline__ int fdiv(int n, const FastDiv& f) {
+  return (int)((__umulhi((unsigned int)n, f.m) + (unsigned int)n) >> f.s);
+}
 
 // Stage s (s = 0 first in the forward transform) has radix radix[s] and acts on
 // sub-sequences of length msize[s] = L / (radix[0] ... radix[s-1]).  Position
 // p = s_0 L/R_0 + s_1 L/(R_0 R_1) + ... holds frequency s_0 + R_0 (s_1 + R_1 (...)).
+// Radices: 2, 3, 4, 5, 6, 8, 9, 10, 12, 15, 16 (host: factor_plan takes the fewest stages).
 struct AxisPlan {
   int L;
   int nst;
   int radix[kMaxStages];
   int msize[kMaxStages];
+  FastDiv dnb[kMaxStages];  // by the stage's butterflies L / R, and by MR = M / R
+  FastDiv dmr[kMaxStages];
 };
 
 template <typename T> struct Cplx;
@@ -128,16 +152,91 @@ __device__ __forceinline__ void dft5(T2* v, bool inv) {
   v[3] = csub(p2, q2);
 }
 
-template <typename T2>
-__device__ __forceinline__ void dft_r(T2* v, int R, bool inv) {
-  switch (R) {
-    case 2: dft2(v); break;
-    case 3: dft3(v, inv); break;
-    case 4: dft4(v, inv); break;
-    case 5: dft5(v, inv); break;
-    case 8: dft8(v, inv); break;
-    default: break;
+// cos and sin of 2 pi k / n for the inner twiddles of the radices 9 (k = 1, 2, 4) and 16 (k = 1, 2, 3, 4, 6, 9)
+__host__ __device__ constexpr double root_cos(int k, int n) {
+  return n == 9 ? (k == 1 ? 0.76604444311897803520 : k == 2 ? 0.17364817766693034885 : -0.93969262078590838405)
+                : (k == 1 ? 0.92387953251128675613 : k == 2 ? 0.70710678118654752440 : k == 3 ? 0.38268343236508977173
+                   : k == 4 ? 0.0 : k == 6 ? -0.70710678118654752440 : -0.92387953251128675613);
+}
+__host__ __device__ constexpr double root_sin(int k, int n) {
+  return n == 9 ? (k == 1 ? 0.64278760968653932632 : k == 2 ? 0.98480775301220805937 : 0.34202014332566873304)
+                : (k == 1 ? 0.38268343236508977173 : k == 2 ? 0.70710678118654752440 : k == 3 ? 0.92387953251128675613
+                   : k == 4 ? 1.0 : k == 6 ? 0.70710678118654752440 : -0.38268343236508977173);
+}
+
+template <int N, typename T2> __device__ __forceinline__ void dft_fixed(T2* v, bool inv);
+
+// DFT of N = P Q coprime factors in registers without twiddles (Good 1958, Thomas 1963): input n = Q n1 + P n2,
+// output k with k = k1 mod P, k = k2 mod Q.
+template <int P, int Q, typename T2>
+__device__ __forceinline__ void dft_coprime(T2* v, bool inv) {
+  constexpr int N = P * Q;
+  T2 y[Q][P];
+#pragma unroll
+  for (int n2 = 0; n2 < Q; ++n2) {
+#pragma unroll
+    for (int n1 = 0; n1 < P; ++n1) y[n2][n1] = v[(Q * n1 + P * n2) % N];
+    dft_fixed<P>(y[n2], inv);
   }
+#pragma unroll
+  for (int k1 = 0; k1 < P; ++k1) {
+    T2 z[Q];
+#pragma unroll
+    for (int n2 = 0; n2 < Q; ++n2) z[n2] = y[n2][k1];
+    dft_fixed<Q>(z, inv);
+#pragma unroll
+    for (int k2 = 0; k2 < Q; ++k2) {
+      int k = k1;
+#pragma unroll
+      for (int s = 0; s < Q; ++s)
+        if (k % Q != k2) k += P;
+      v[k] = z[k2];
+    }
+  }
+}
+// DFT of N = P P (9, 16) in registers: n = P n1 + n2, k = k1 + P k2, twiddles w_N^{n2 k1}.
+template <int P, typename T2>
+__device__ __forceinline__ void dft_square(T2* v, bool inv) {
+  typedef decltype(T2::x) T;
+  constexpr int N = P * P;
+  T2 y[P][P];
+#pragma unroll
+  for (int n2 = 0; n2 < P; ++n2) {
+#pragma unroll
+    for (int n1 = 0; n1 < P; ++n1) y[n2][n1] = v[P * n1 + n2];
+    dft_fixed<P>(y[n2], inv);
+  }
+#pragma unroll
+  for (int k1 = 0; k1 < P; ++k1) {
+    T2 z[P];
+#pragma unroll
+    for (int n2 = 0; n2 < P; ++n2) {
+      z[n2] = y[n2][k1];
+      if (n2 * k1 > 0) {
+        const T c = (T)root_cos(n2 * k1, N), sn = (T)root_sin(n2 * k1, N);
+        const T2 a = z[n2];
+        z[n2] = inv ? cmk<T2>(a.x * c - a.y * sn, a.x * sn + a.y * c) : cmk<T2>(a.x * c + a.y * sn, a.y * c - a.x * sn);
+      }
+    }
+    dft_fixed<P>(z, inv);
+#pragma unroll
+    for (int k2 = 0; k2 < P; ++k2) v[k1 + P * k2] = z[k2];
+  }
+}
+
+template <int N, typename T2>
+__device__ __forceinline__ void dft_fixed(T2* v, bool inv) {
+  if constexpr (N == 2) dft2(v);
+  else if constexpr (N == 3) dft3(v, inv);
+  else if constexpr (N == 4) dft4(v, inv);
+  else if constexpr (N == 5) dft5(v, inv);
+  else if constexpr (N == 6) dft_coprime<2, 3>(v, inv);
+  else if constexpr (N == 8) dft8(v, inv);
+  else if constexpr (N == 9) dft_square<3>(v, inv);
+  else if constexpr (N == 10) dft_coprime<2, 5>(v, inv);
+  else if constexpr (N == 12) dft_coprime<3, 4>(v, inv);
+  else if constexpr (N == 15) dft_coprime<3, 5>(v, inv);
+  else if constexpr (N == 16) dft_square<4>(v, inv);
 }
 
 // Tiles of x1-lines (few columns, an odd row stride) pad one row every 16 rows,
@@ -151,28 +250,6 @@ constexpr int kPadShift = 4;
 __host__ __device__ constexpr int pad_row(int e) { return e + (e >> kPadShift); }
 __host__ __device__ constexpr int padded_rows(int n) { return n + ((n + (1 << kPadShift) - 1) >> kPadShift); }
 __device__ __forceinline__ int prow(int e, int pad) { return pad ? pad_row(e) : e; }
-
-// Division by a runtime divisor 1 <= d < 2^31 through a multiply-high and a
-// shift (Granlund and Montgomery 1994), exact for 0 <= n < 2^31.
-struct FastDiv {
-  unsigned int m, s;
-  int d;
-};
-
-__host__ __device__ inline FastDiv make_fastdiv(int d) {
-  unsigned int l = 0;
-  while ((1u << l) < (unsigned int)d) ++l;
-  const unsigned long long m = ((1ull << 32) * ((1ull << l) - (unsigned long long)d)) / (unsigned long long)d + 1ull;
-  FastDiv f;
-  f.m = (unsigned int)m;
-  f.s = l;
-  f.d = d;
-  return f;
-}
-
-__device__ __forceinline__ int fdiv(int n, const FastDiv& f) {
-  return (int)((__umulhi((unsigned int)n, f.m) + (unsigned int)n) >> f.s);
-}
 
 // Radix plan of a power-of-two length, identical to the host plan: radix 8
 // stages, led by one radix-4 stage (log2 L = 2 mod 3), two radix-4 stages
@@ -192,11 +269,11 @@ __host__ __device__ constexpr int p2_msize(int L, int s) { return s == 0 ? L : p
 // Lengths whose transforms run the compile-time stages (tile_fft_ct).
 __host__ __device__ constexpr bool ct_length(int L) { return L == 64 || L == 128 || L == 256 || L == 512; }
 // Radix-3 lengths whose strided (x2 / x3) transforms also run compile-time stages, with the host plan:
-// the power-of-two plan of L / 3, then one radix-3 stage (48 = 4 4 3, 96 = 4 8 3).
+// 48 = 8 6, 96 = 8 12 (two shared-memory stages; the last one, M = R, needs no twiddle rows).
 __host__ __device__ constexpr bool r3_length(int L) { return L == 48 || L == 96; }
-__host__ __device__ constexpr int ct_nst(int L) { return r3_length(L) ? p2_nst(L / 3) + 1 : p2_nst(L); }
+__host__ __device__ constexpr int ct_nst(int L) { return r3_length(L) ? 2 : p2_nst(L); }
 __host__ __device__ constexpr int ct_radix(int L, int s) {
-  return r3_length(L) ? (s < p2_nst(L / 3) ? p2_radix(L / 3, s) : 3) : p2_radix(L, s);
+  return r3_length(L) ? (s == 0 ? 8 : L / 8) : p2_radix(L, s);
 }
 __host__ __device__ constexpr int ct_msize(int L, int s) { return s == 0 ? L : ct_msize(L, s - 1) / ct_radix(L, s - 1); }
 // Twiddle table of a compile-time length, laid out by stage (read by the
@@ -229,7 +306,7 @@ __host__ __device__ constexpr int strided_tw_offset(int L, int s) {
 // that a kernel pays no run-time recursion for it.
 __host__ __device__ constexpr int tw_count(int L, int layout) {
   return layout == kTwX1 ? (L == 64 ? 64 : L == 128 ? 160 : L == 256 ? 320 : L == 512 ? 576 : ((L + 1) & ~1))
-       : layout == kTwStrided ? (L == 48 ? 60 : L == 64 ? 80 : L == 96 ? 126 : L == 128 ? 160 : L == 256 ? 336
+       : layout == kTwStrided ? (L == 48 ? 60 : L == 64 ? 80 : L == 96 ? 120 : L == 128 ? 160 : L == 256 ? 336
                                  : L == 512 ? 720 : ((L + 1) & ~1))
        : ((L + 1) & ~1);
 }
@@ -245,74 +322,6 @@ static_assert(tw_count(48, kTwStrided) == strided_tw_offset(48, ct_nst(48)) &&
                   tw_count(256, kTwStrided) == strided_tw_offset(256, p2_nst(256)) &&
                   tw_count(512, kTwStrided) == strided_tw_offset(512, p2_nst(512)),
               "strided twiddle counts");
-
-template <int R, typename T2>
-__device__ __forceinline__ void dft_fixed(T2* v, bool inv) {
-  if (R == 2) dft2(v);
-  else if (R == 3) dft3(v, inv);
-  else if (R == 4) dft4(v, inv);
-  else dft8(v, inv);
-}
-
-template <int L, int S, typename T2>
-__device__ __forceinline__ void p2_stage(T2* buf, int nblk, int BS, int C, const FastDiv& fc, int ncols, const T2* tw,
-                                         bool inv, int pad) {
-  constexpr int R = p2_radix(L, S);
-  constexpr int M = p2_msize(L, S);
-  constexpr int MR = M / R;
-  constexpr int NB = L / R;
-  constexpr int TSTR = L / M;
-  const int total = nblk * NB * ncols;
-  const int rs = MR * C;
-  for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
-    const int rest = fdiv(idx, fc);
-    const int c = idx - rest * ncols;
-    const int bf = rest & (NB - 1);
-    const int blk = rest / NB;
-    const int b = bf / MR, j = bf & (MR - 1);
-    T2* base = buf + blk * BS + c;
-    const int e0 = b * M + j;
-    int off[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) off[r] = pad ? prow(e0 + r * MR, 1) * C : (e0 * C + r * rs);
-    T2 v[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = base[off[r]];
-    if (!inv) {
-      dft_fixed<R>(v, false);
-      if (MR > 1 && j) {
-#pragma unroll
-        for (int r = 1; r < R; ++r) v[r] = cmul(v[r], tw[j * r * TSTR]);
-      }
-    } else {
-      if (MR > 1 && j) {
-#pragma unroll
-        for (int r = 1; r < R; ++r) v[r] = cmulc(v[r], tw[j * r * TSTR]);
-      }
-      dft_fixed<R>(v, true);
-    }
-#pragma unroll
-    for (int r = 0; r < R; ++r) base[off[r]] = v[r];
-  }
-  __syncthreads();
-}
-
-template <int L, typename T2>
-__device__ void tile_fft_p2(T2* buf, int nblk, int BS, int C, int ncols, const T2* tw, bool inv, int pad) {
-  constexpr int NST = p2_nst(L);
-  const FastDiv fc = make_fastdiv(ncols);
-  if (!inv) {
-    if constexpr (NST > 0) p2_stage<L, 0>(buf, nblk, BS, C, fc, ncols, tw, false, pad);
-    if constexpr (NST > 1) p2_stage<L, 1>(buf, nblk, BS, C, fc, ncols, tw, false, pad);
-    if constexpr (NST > 2) p2_stage<L, 2>(buf, nblk, BS, C, fc, ncols, tw, false, pad);
-    if constexpr (NST > 3) p2_stage<L, 3>(buf, nblk, BS, C, fc, ncols, tw, false, pad);
-  } else {
-    if constexpr (NST > 3) p2_stage<L, 3>(buf, nblk, BS, C, fc, ncols, tw, true, pad);
-    if constexpr (NST > 2) p2_stage<L, 2>(buf, nblk, BS, C, fc, ncols, tw, true, pad);
-    if constexpr (NST > 1) p2_stage<L, 1>(buf, nblk, BS, C, fc, ncols, tw, true, pad);
-    if constexpr (NST > 0) p2_stage<L, 0>(buf, nblk, BS, C, fc, ncols, tw, true, pad);
-  }
-}
 
 // One twiddle row of the stage layout (R complex values, 16-byte aligned) into
 // registers: 16-byte loads for FP32, one load per value for FP64.
@@ -445,74 +454,102 @@ __device__ __forceinline__ void tile_fft_p2_ct(T2* buf, int nblk, const T2* tw, 
   }
 }
 
-// Mixed-radix transform for any supported length (runtime plan).
-template <typename T2>
-__device__ void tile_fft_generic(T2* buf, int nblk, int BS, int C, int ncols, const AxisPlan& p, const T2* tw, bool inv,
-                                 int pad) {
-  const int L = p.L;
-  for (int si = 0; si < p.nst; ++si) {
-    const int s = inv ? p.nst - 1 - si : si;
-    const int R = p.radix[s];
-    const int M = p.msize[s];
-    const int MR = M / R;
-    const int tstr = L / M;
-    const int nb = L / R;
-    const int total = nblk * nb * ncols;
-    const int rs = MR * C;
-    for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
-      const int c = idx % ncols;
-      const int rest = idx / ncols;
-      const int bf = rest % nb;
-      const int blk = rest / nb;
-      const int b = bf / MR, j = bf - b * MR;
-      T2* base = buf + blk * BS + c;
-      const int e0 = b * M + j;
-      T2 v[kMaxRadix];
+// One stage of radix R of the run-time plan on a tile of nblk blocks (row stride C, the first NCOLS columns
+// transformed, rows padded when PAD).  LC > 0: the length, so that every index division is by a constant.
+template <int R, int LC, int MC, int C, int NCOLS, bool PAD, bool INV, typename T2>
+__device__ __forceinline__ void gen_stage(T2* buf, int nblk, int BS, const AxisPlan& p, int s, const T2* tw) {
+  const int L = LC ? LC : p.L;
+  const int M = LC ? MC : p.msize[s];
+  const int MR = LC ? MC / R : p.dmr[s].d;
+  const int nb = LC ? LC / R : p.dnb[s].d;
+  const int tstr = LC ? LC / MC : L / M;
+  const int total = nblk * nb * NCOLS;
+  FastDiv dnb = {0u, 0u, 1}, dmr = {0u, 0u, 1};
+  if (!LC) {
+    dnb = p.dnb[s];
+    dmr = p.dmr[s];
+  }
+  for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
+    const int rest = (int)((unsigned)idx / (unsigned)NCOLS), c = idx - rest * NCOLS;
+    const int blk = LC ? (int)((unsigned)rest / (unsigned)(LC ? LC / R : 1)) : fdiv(rest, dnb), bf = rest - blk * nb;
+    const int b = LC ? (int)((unsigned)bf / (unsigned)(LC ? MC / R : 1)) : fdiv(bf, dmr), j = bf - b * MR;
+    T2* base = buf + blk * BS + c;
+    const int e0 = b * M + j;
+    T2 v[R];
 #pragma unroll
-      for (int r = 0; r < kMaxRadix; ++r)
-        if (r < R) v[r] = base[pad ? prow(e0 + r * MR, 1) * C : e0 * C + r * rs];
-      if (!inv) {
-        dft_r(v, R, false);
-        if (j) {
+    for (int r = 0; r < R; ++r) v[r] = base[prow(e0 + r * MR, PAD) * C];
+    if (!INV) dft_fixed<R>(v, false);
+    if (MR > 1) {
+      const T2* w = tw;
 #pragma unroll
-          for (int r = 1; r < kMaxRadix; ++r)
-            if (r < R) v[r] = cmul(v[r], tw[j * r * tstr]);
-        }
-      } else {
-        if (j) {
-#pragma unroll
-          for (int r = 1; r < kMaxRadix; ++r)
-            if (r < R) v[r] = cmulc(v[r], tw[j * r * tstr]);
-        }
-        dft_r(v, R, true);
+      for (int r = 1; r < R; ++r) {
+        w += j * tstr;
+        v[r] = INV ? cmulc(v[r], *w) : cmul(v[r], *w);
       }
-#pragma unroll
-      for (int r = 0; r < kMaxRadix; ++r)
-        if (r < R) base[pad ? prow(e0 + r * MR, 1) * C : e0 * C + r * rs] = v[r];
     }
-    __syncthreads();
+    if (INV) dft_fixed<R>(v, true);
+#pragma unroll
+    for (int r = 0; r < R; ++r) base[prow(e0 + r * MR, PAD) * C] = v[r];
+  }
+  __syncthreads();
+}
+
+// Mixed-radix transform for any supported length (runtime plan).
+template <int C, int NCOLS, bool PAD, bool INV, typename T2>
+__device__ __forceinline__ void tile_fft_generic(T2* buf, int nblk, int BS, const AxisPlan& p, const T2* tw) {
+  for (int si = 0; si < p.nst; ++si) {
+    const int s = INV ? p.nst - 1 - si : si;
+    switch (p.radix[s]) {
+#define FFTLS_GEN(R) \
+  case R: gen_stage<R, 0, 0, C, NCOLS, PAD, INV>(buf, nblk, BS, p, s, tw); break
+      FFTLS_GEN(2);
+      FFTLS_GEN(3);
+      FFTLS_GEN(4);
+      FFTLS_GEN(5);
+      FFTLS_GEN(6);
+      FFTLS_GEN(8);
+      FFTLS_GEN(9);
+      FFTLS_GEN(10);
+      FFTLS_GEN(12);
+      FFTLS_GEN(15);
+      FFTLS_GEN(16);
+#undef FFTLS_GEN
+      default: break;
+    }
   }
 }
 
-// In-place transform of a tile (see the file comment) with a runtime tile
-// geometry, for the lengths tile_fft_ct does not specialise: the short and the
-// longest powers of two run their fixed plans, any other length the runtime
-// plan.  tw[t] = e^{-2 pi i t / L} (shared memory).  Ends with __syncthreads()
-// when the length has at least one stage.  pad = 1: row e of the tile is stored
-// at prow(e) (x1-line tiles).
-template <typename T2>
-__device__ void tile_fft_rt(T2* buf, int nblk, int BS, int C, int ncols, const AxisPlan& p, const T2* tw, bool inv,
-                            int pad) {
-  switch (p.L) {
-    case 1: return;
-    case 2: tile_fft_p2<2>(buf, nblk, BS, C, ncols, tw, inv, pad); return;
-    case 4: tile_fft_p2<4>(buf, nblk, BS, C, ncols, tw, inv, pad); return;
-    case 8: tile_fft_p2<8>(buf, nblk, BS, C, ncols, tw, inv, pad); return;
-    case 16: tile_fft_p2<16>(buf, nblk, BS, C, ncols, tw, inv, pad); return;
-    case 32: tile_fft_p2<32>(buf, nblk, BS, C, ncols, tw, inv, pad); return;
-    case 1024: tile_fft_p2<1024>(buf, nblk, BS, C, ncols, tw, inv, pad); return;
-    default: tile_fft_generic(buf, nblk, BS, C, ncols, p, tw, inv, pad); return;
+// Two stages R0, R1 of the length R0 R1 (the host plan's), every index constant.
+template <int R0, int R1, int C, int NCOLS, bool PAD, bool INV, typename T2>
+__device__ __forceinline__ void tile_fft_two(T2* buf, int nblk, int BS, const AxisPlan& p, const T2* tw) {
+  if (INV) {
+    gen_stage<R1, R0 * R1, R1, C, NCOLS, PAD, true>(buf, nblk, BS, p, 1, tw);
+    gen_stage<R0, R0 * R1, R0 * R1, C, NCOLS, PAD, true>(buf, nblk, BS, p, 0, tw);
+  } else {
+    gen_stage<R0, R0 * R1, R0 * R1, C, NCOLS, PAD, false>(buf, nblk, BS, p, 0, tw);
+    gen_stage<R1, R0 * R1, R1, C, NCOLS, PAD, false>(buf, nblk, BS, p, 1, tw);
   }
+}
+
+// In-place transform of a tile (see the file comment) for the lengths without stages of their own in tile_fft_ct or
+// tile_fft_strided: 24, 32 and, in the x1 tiles, 48 and 96 run two constant stages, any other length its plan.
+// tw[t] = e^{-2 pi i t / L} (shared memory).  Ends with __syncthreads() when the length has at least one stage.
+// PAD: row e of the tile is stored at prow(e) (x1-line tiles).
+template <int C, int NCOLS, bool PAD, bool INV, typename T2>
+__device__ __forceinline__ void tile_fft_rt(T2* buf, int nblk, int BS, const AxisPlan& p, const T2* tw) {
+  switch (p.L) {
+    case 24: tile_fft_two<4, 6, C, NCOLS, PAD, INV>(buf, nblk, BS, p, tw); return;
+    case 32: tile_fft_two<4, 8, C, NCOLS, PAD, INV>(buf, nblk, BS, p, tw); return;
+    case 48: if constexpr (PAD) { tile_fft_two<8, 6, C, NCOLS, PAD, INV>(buf, nblk, BS, p, tw); return; } break;
+    case 96: if constexpr (PAD) { tile_fft_two<8, 12, C, NCOLS, PAD, INV>(buf, nblk, BS, p, tw); return; } break;
+    default: break;
+  }
+  tile_fft_generic<C, NCOLS, PAD, INV>(buf, nblk, BS, p, tw);
+}
+// the same as a call, for the separate x1 passes (once per run of iterations)
+template <int C, int NCOLS, bool PAD, bool INV, typename T2>
+__device__ __noinline__ void tile_fft_rt_call(T2* buf, int nblk, int BS, const AxisPlan& p, const T2* tw) {
+  tile_fft_rt<C, NCOLS, PAD, INV>(buf, nblk, BS, p, tw);
 }
 
 // Stage S of the length-L transform on a strided tile (x2 / x3 passes): one
@@ -660,18 +697,24 @@ __device__ __forceinline__ void strided_fft(T2* buf, const T2* tw) {
 template <typename T2>
 __host__ __device__ constexpr bool strided_fits(int L, int C) { return (long long)L * C * (long long)sizeof(T2) <= 232448; }
 
-template <int C, int NT, bool INV, bool PAIR, typename T2>
-__device__ void tile_fft_strided(T2* buf, const AxisPlan& p, const T2* tw) {
-  switch (p.L) {
-    case 48: if constexpr (strided_fits<T2>(48, C)) { strided_fft<48, C, NT, INV, PAIR>(buf, tw); return; } break;
-    case 64: if constexpr (strided_fits<T2>(64, C)) { strided_fft<64, C, NT, INV, PAIR>(buf, tw); return; } break;
-    case 96: if constexpr (strided_fits<T2>(96, C)) { strided_fft<96, C, NT, INV, PAIR>(buf, tw); return; } break;
-    case 128: if constexpr (strided_fits<T2>(128, C)) { strided_fft<128, C, NT, INV, PAIR>(buf, tw); return; } break;
-    case 256: if constexpr (strided_fits<T2>(256, C)) { strided_fft<256, C, NT, INV, PAIR>(buf, tw); return; } break;
-    case 512: if constexpr (strided_fits<T2>(512, C)) { strided_fft<512, C, NT, INV, PAIR>(buf, tw); return; } break;
-    default: break;
+// CT: the lengths with compile-time stages (strided_ct_length); else any other (kernels of their own, so that neither
+// pays for the other's registers).
+__host__ __device__ constexpr bool strided_ct_length(int L) { return ct_length(L) || r3_length(L); }
+template <int C, int NT, bool INV, bool PAIR, bool CT, typename T2>
+__device__ __forceinline__ void tile_fft_strided(T2* buf, const AxisPlan& p, const T2* tw) {
+  if constexpr (CT) {
+    switch (p.L) {
+      case 48: if constexpr (strided_fits<T2>(48, C)) strided_fft<48, C, NT, INV, PAIR>(buf, tw); break;
+      case 64: if constexpr (strided_fits<T2>(64, C)) strided_fft<64, C, NT, INV, PAIR>(buf, tw); break;
+      case 96: if constexpr (strided_fits<T2>(96, C)) strided_fft<96, C, NT, INV, PAIR>(buf, tw); break;
+      case 128: if constexpr (strided_fits<T2>(128, C)) strided_fft<128, C, NT, INV, PAIR>(buf, tw); break;
+      case 256: if constexpr (strided_fits<T2>(256, C)) strided_fft<256, C, NT, INV, PAIR>(buf, tw); break;
+      case 512: if constexpr (strided_fits<T2>(512, C)) strided_fft<512, C, NT, INV, PAIR>(buf, tw); break;
+      default: break;
+    }
+  } else {
+    tile_fft_rt<C, C, false, INV>(buf, 1, 0, p, tw);
   }
-  tile_fft_rt(buf, 1, 0, C, C, p, tw, INV, 0);
 }
 
 // tile_fft with the tile geometry fixed at compile time (row stride C complex
@@ -680,15 +723,19 @@ __device__ void tile_fft_strided(T2* buf, const AxisPlan& p, const T2* tw) {
 // length the runtime paths.  BS is the block stride of the general path.  tw
 // holds tw_count(L, PAD) entries: the padded (x1) tiles of the compile-time
 // lengths read the stage layout, every other transform the plain table.
-template <int C, int NCOLS, bool PAD, typename T2>
-__device__ void tile_fft_ct(T2* buf, int nblk, int BS, const AxisPlan& p, const T2* tw, bool inv) {
+// CALL: the other lengths through tile_fft_rt_call.
+template <int C, int NCOLS, bool PAD, bool INV, bool CALL, typename T2>
+__device__ __forceinline__ void tile_fft_ct(T2* buf, int nblk, int BS, const AxisPlan& p, const T2* tw) {
   static_assert(ct_length(64) && ct_length(128) && ct_length(256) && ct_length(512), "compile-time lengths");
   switch (p.L) {
-    case 64: tile_fft_p2_ct<64, C, NCOLS, PAD>(buf, nblk, tw, inv); return;
-    case 128: tile_fft_p2_ct<128, C, NCOLS, PAD>(buf, nblk, tw, inv); return;
-    case 256: tile_fft_p2_ct<256, C, NCOLS, PAD>(buf, nblk, tw, inv); return;
-    case 512: tile_fft_p2_ct<512, C, NCOLS, PAD>(buf, nblk, tw, inv); return;
-    default: tile_fft_rt(buf, nblk, BS, C, NCOLS, p, tw, inv, PAD ? 1 : 0); return;
+    case 64: tile_fft_p2_ct<64, C, NCOLS, PAD>(buf, nblk, tw, INV); return;
+    case 128: tile_fft_p2_ct<128, C, NCOLS, PAD>(buf, nblk, tw, INV); return;
+    case 256: tile_fft_p2_ct<256, C, NCOLS, PAD>(buf, nblk, tw, INV); return;
+    case 512: tile_fft_p2_ct<512, C, NCOLS, PAD>(buf, nblk, tw, INV); return;
+    default:
+      if constexpr (CALL) tile_fft_rt_call<C, NCOLS, PAD, INV>(buf, nblk, BS, p, tw);
+      else tile_fft_rt<C, NCOLS, PAD, INV>(buf, nblk, BS, p, tw);
+      return;
   }
 }
 

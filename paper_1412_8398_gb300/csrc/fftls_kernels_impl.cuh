@@ -482,7 +482,7 @@ __device__ __forceinline__ void k_fwd_x_body(const IterArgs<T>& a, const AxisPla
       const long long ln = l0 + (long long)gridDim.x * G;
       if (ln < nlines) prefetch_voxels<T>(a.eps, a.phase, g.N, NC, ln * L1, (int)min((long long)G, nlines - ln) * L1);
     }
-    tile_fft_ct<CP, NP, true>(tile, nl, BS, pl[0], tws, false);
+    tile_fft_ct<CP, NP, true, false, true>(tile, nl, BS, pl[0], tws);
     fwd_x_untangle<T, DIM, DUAL>(a, tile, nl, l0, BS, fH);
     __syncthreads();
   }
@@ -606,7 +606,7 @@ __device__ __forceinline__ void k_fwd_x_staged_body(const IterArgs<float>& a, co
       fence_async_shared();
       issue(l0 + step);
     }
-    tile_fft_ct<CP, NP, true>(tile, nl, BS, pl[0], tws, false);
+    tile_fft_ct<CP, NP, true, false, true>(tile, nl, BS, pl[0], tws);
     fwd_x_untangle<T, DIM, DUAL>(a, tile, nl, l0, BS, fH);
     __syncthreads();
   }
@@ -828,7 +828,7 @@ __global__ void __launch_bounds__(kEThreads) k_eta_stencil(const __grid_constant
 // hold fewer modes, its other columns are transformed but never stored).
 // Blocks of strided_threads(W) threads (a compile-time count for the stages).
 
-template <typename T, int NC, int W>
+template <typename T, int NC, int W, bool CT>
 __device__ __forceinline__ void k_mid_y_body(const IterArgs<T>& a, const AxisPlan* pl, int inv, int kind) {
   typedef typename Cplx<T>::type T2;
   constexpr int NT = strided_threads(W);
@@ -844,21 +844,21 @@ __device__ __forceinline__ void k_mid_y_body(const IterArgs<T>& a, const AxisPla
   const long long base = ((long long)blockIdx.y * n2 * g.H + x0) * NC;
   const long long rstride = (long long)g.H * NC;
   if (!tile_load<C, false>(tile, spec + base, rstride, n2, cols, a.ctrl)) return;
-  if (inv) tile_fft_strided<C, NT, true, false>(tile, pl[1], tws);
-  else tile_fft_strided<C, NT, false, true>(tile, pl[1], tws);
+  if (inv) tile_fft_strided<C, NT, true, false, CT>(tile, pl[1], tws);
+  else tile_fft_strided<C, NT, false, true, CT>(tile, pl[1], tws);
   tile_store<C, false>(tile, spec + base, rstride, n2, cols);
 }
 
 // GRP: a grouped launch (fftls_solve_batched), every block working on its sample's view
-template <typename T, int NC, int W, bool GRP>
+template <typename T, int NC, int W, bool CT, bool GRP>
 __global__ void __launch_bounds__(strided_threads(W)) k_mid_y(const __grid_constant__ IterArgs<T> a_, int inv) {
   if constexpr (GRP) {
     const int kinds = gridDim.z / a_.nsmp;
     IterArgs<T> a = a_;
     at_sample(a, blockIdx.z / kinds);
-    k_mid_y_body<T, NC, W>(a, a_.pl, inv, (int)(blockIdx.z % kinds));
+    k_mid_y_body<T, NC, W, CT>(a, a_.pl, inv, (int)(blockIdx.z % kinds));
   } else {
-    k_mid_y_body<T, NC, W>(a_, a_.pl, inv, (int)blockIdx.z);
+    k_mid_y_body<T, NC, W, CT>(a_, a_.pl, inv, (int)blockIdx.z);
   }
 }
 
@@ -1171,7 +1171,7 @@ __device__ __forceinline__ void store_mode6(double2* p, const double2 (&X)[6]) {
 // transformed, no eta here): the modes take green_rd_mode with the per-axis
 // factors of rd (by storage position), kr_1 = a_1 b_2 b_3, kr_2 = b_1 a_2 b_3,
 // kr_3 = b_1 b_2 a_3.  Otherwise the general fourier_mode.
-template <typename T, int DIM, int W, bool FAST>
+template <typename T, int DIM, int W, bool FAST, bool CT>
 __device__ __forceinline__ void k_fourier_z_body(const IterArgs<T>& a, const AxisPlan* pl, int kind) {
   typedef typename Cplx<T>::type T2;
   constexpr int NC = Comp<DIM>::NC;
@@ -1196,7 +1196,7 @@ __device__ __forceinline__ void k_fourier_z_body(const IterArgs<T>& a, const Axi
   const long long base = ((long long)py * g.H + x0) * NC;
   const long long zstride = (DIM == 3 ? (long long)g.n2 : 1LL) * g.H * NC;
   if (!tile_load<C, true>(tile, spec + base, zstride, nl, cols, a.ctrl)) return;
-  tile_fft_strided<C, NT, false, false>(tile, pl[AX], tws);
+  tile_fft_strided<C, NT, false, false, CT>(tile, pl[AX], tws);
   T eta_acc = (T)0;
   if constexpr (FAST) {
     static_assert(DIM == 3 && NT % W == 0, "fast Fourier pass: 3D, whole modes per thread");
@@ -1243,7 +1243,7 @@ __device__ __forceinline__ void k_fourier_z_body(const IterArgs<T>& a, const Axi
   }
   __syncthreads();
   if (do_green) {
-    tile_fft_strided<C, NT, true, false>(tile, pl[AX], tws);
+    tile_fft_strided<C, NT, true, false, CT>(tile, pl[AX], tws);
     tile_store<C, true>(tile, spec + base, zstride, nl, cols);
   }
   if (!a.eta_real) {  // with the real-space eta the x1 pass owns part_eta
@@ -1255,15 +1255,15 @@ __device__ __forceinline__ void k_fourier_z_body(const IterArgs<T>& a, const Axi
 }
 
 // GRP: a grouped launch (fftls_solve_batched), every block working on its sample's view
-template <typename T, int DIM, int W, bool FAST, bool GRP>
+template <typename T, int DIM, int W, bool FAST, bool CT, bool GRP>
 __global__ void __launch_bounds__(strided_threads(W)) k_fourier_z(const __grid_constant__ IterArgs<T> a_) {
   if constexpr (GRP) {
     const int kinds = gridDim.z / a_.nsmp;
     IterArgs<T> a = a_;
     at_sample(a, blockIdx.z / kinds);
-    k_fourier_z_body<T, DIM, W, FAST>(a, a_.pl, (int)(blockIdx.z % kinds));
+    k_fourier_z_body<T, DIM, W, FAST, CT>(a, a_.pl, (int)(blockIdx.z % kinds));
   } else {
-    k_fourier_z_body<T, DIM, W, FAST>(a_, a_.pl, (int)blockIdx.z);
+    k_fourier_z_body<T, DIM, W, FAST, CT>(a_, a_.pl, (int)blockIdx.z);
   }
 }
 
@@ -1470,7 +1470,7 @@ __device__ __forceinline__ void k_inv_x_body(const IterArgs<T>& a, const AxisPla
           asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(base) + off));
       }
     }
-    tile_fft_ct<CP, NPI, true>(tile, nl, BS, pl[0], tws, true);
+    tile_fft_ct<CP, NPI, true, true, true>(tile, nl, BS, pl[0], tws);
     if (stage) {
       bool done = false;
       for (long long k = 0; k < kBulkWaitRounds && !done; ++k) done = mbar_try_wait(bar, parity);
@@ -1725,7 +1725,9 @@ template <typename T, bool GRP>
 cudaError_t launch_mid_y_t(const IterArgs<T>& a, bool inv, cudaStream_t s) {
   if (a.dim == 2 || a.g.n2 == 1) return cudaSuccess;  // 2D: the Fourier pass transforms along x2
   dim3 grid((a.g.H + a.y_w - 1) / a.y_w, a.g.n3, ((!inv && a.dual && !a.eta_real) ? 2 : 1) * (GRP ? a.nsmp : 1));
-#define FFTLS_MIDY(NCV, WV) k_mid_y<T, NCV, WV, GRP><<<grid, strided_threads(WV), a.y_smem, s>>>(a, inv ? 1 : 0)
+  const bool ct = strided_ct_length(a.g.n2);
+#define FFTLS_MIDY(NCV, WV)                                                                             \
+  (ct ? k_mid_y<T, NCV, WV, true, GRP> : k_mid_y<T, NCV, WV, false, GRP>)<<<grid, strided_threads(WV), a.y_smem, s>>>(a, inv ? 1 : 0)
 #define FFTLS_MIDY_W(NCV)                                                                               \
   switch (a.y_w) {                                                                                      \
     case 1: FFTLS_MIDY(NCV, 1); break;                                                                  \
@@ -1750,7 +1752,9 @@ bool fourier_fast(const IterArgs<T>& a) {
 template <typename T, bool GRP>
 cudaError_t launch_fourier_z_t(const IterArgs<T>& a, cudaStream_t s) {
   dim3 grid((a.g.H + a.z_w - 1) / a.z_w, a.dim == 3 ? a.g.n2 : 1, ((a.dual && !a.eta_real) ? 2 : 1) * (GRP ? a.nsmp : 1));
-#define FFTLS_FZ(D, WV, F) k_fourier_z<T, D, WV, F, GRP><<<grid, strided_threads(WV), a.z_smem, s>>>(a)
+  const bool ct = strided_ct_length(a.dim == 3 ? a.g.n3 : a.g.n2);
+#define FFTLS_FZ(D, WV, F)                                                                              \
+  (ct ? k_fourier_z<T, D, WV, F, true, GRP> : k_fourier_z<T, D, WV, F, false, GRP>)<<<grid, strided_threads(WV), a.z_smem, s>>>(a)
 #define FFTLS_FZ_W(D, F)                                                                                \
   switch (a.z_w) {                                                                                      \
     case 1: FFTLS_FZ(D, 1, F); break;                                                                   \
@@ -1834,33 +1838,53 @@ template <typename T> cudaError_t launch_reduce_delta(const IterArgs<T>& a, cuda
 template <typename T, bool GRP>
 cudaError_t set_attrs_y_t(size_t smax) {
   cudaError_t e = cudaSuccess;
-  FFTLS_ATTR((k_mid_y<T, 6, 1, GRP>));
-  FFTLS_ATTR((k_mid_y<T, 6, 2, GRP>));
-  FFTLS_ATTR((k_mid_y<T, 6, 4, GRP>));
-  FFTLS_ATTR((k_mid_y<T, 6, 8, GRP>));
-  FFTLS_ATTR((k_mid_y<T, 6, 16, GRP>));
+  FFTLS_ATTR((k_mid_y<T, 6, 1, true, GRP>));
+  FFTLS_ATTR((k_mid_y<T, 6, 1, false, GRP>));
+  FFTLS_ATTR((k_mid_y<T, 6, 2, true, GRP>));
+  FFTLS_ATTR((k_mid_y<T, 6, 2, false, GRP>));
+  FFTLS_ATTR((k_mid_y<T, 6, 4, true, GRP>));
+  FFTLS_ATTR((k_mid_y<T, 6, 4, false, GRP>));
+  FFTLS_ATTR((k_mid_y<T, 6, 8, true, GRP>));
+  FFTLS_ATTR((k_mid_y<T, 6, 8, false, GRP>));
+  FFTLS_ATTR((k_mid_y<T, 6, 16, true, GRP>));
+  FFTLS_ATTR((k_mid_y<T, 6, 16, false, GRP>));
   return e;
 }
 
 template <typename T, bool GRP>
 cudaError_t set_attrs_z_t(size_t smax) {
   cudaError_t e = cudaSuccess;
-  FFTLS_ATTR((k_fourier_z<T, 3, 1, false, GRP>));
-  FFTLS_ATTR((k_fourier_z<T, 3, 2, false, GRP>));
-  FFTLS_ATTR((k_fourier_z<T, 3, 4, false, GRP>));
-  FFTLS_ATTR((k_fourier_z<T, 3, 8, false, GRP>));
-  FFTLS_ATTR((k_fourier_z<T, 3, 16, false, GRP>));
-  FFTLS_ATTR((k_fourier_z<T, 3, 1, true, GRP>));
-  FFTLS_ATTR((k_fourier_z<T, 3, 2, true, GRP>));
-  FFTLS_ATTR((k_fourier_z<T, 3, 4, true, GRP>));
-  FFTLS_ATTR((k_fourier_z<T, 3, 8, true, GRP>));
-  FFTLS_ATTR((k_fourier_z<T, 3, 16, true, GRP>));
+  FFTLS_ATTR((k_fourier_z<T, 3, 1, false, true, GRP>));
+  FFTLS_ATTR((k_fourier_z<T, 3, 1, false, false, GRP>));
+  FFTLS_ATTR((k_fourier_z<T, 3, 2, false, true, GRP>));
+  FFTLS_ATTR((k_fourier_z<T, 3, 2, false, false, GRP>));
+  FFTLS_ATTR((k_fourier_z<T, 3, 4, false, true, GRP>));
+  FFTLS_ATTR((k_fourier_z<T, 3, 4, false, false, GRP>));
+  FFTLS_ATTR((k_fourier_z<T, 3, 8, false, true, GRP>));
+  FFTLS_ATTR((k_fourier_z<T, 3, 8, false, false, GRP>));
+  FFTLS_ATTR((k_fourier_z<T, 3, 16, false, true, GRP>));
+  FFTLS_ATTR((k_fourier_z<T, 3, 16, false, false, GRP>));
+  FFTLS_ATTR((k_fourier_z<T, 3, 1, true, true, GRP>));
+  FFTLS_ATTR((k_fourier_z<T, 3, 1, true, false, GRP>));
+  FFTLS_ATTR((k_fourier_z<T, 3, 2, true, true, GRP>));
+  FFTLS_ATTR((k_fourier_z<T, 3, 2, true, false, GRP>));
+  FFTLS_ATTR((k_fourier_z<T, 3, 4, true, true, GRP>));
+  FFTLS_ATTR((k_fourier_z<T, 3, 4, true, false, GRP>));
+  FFTLS_ATTR((k_fourier_z<T, 3, 8, true, true, GRP>));
+  FFTLS_ATTR((k_fourier_z<T, 3, 8, true, false, GRP>));
+  FFTLS_ATTR((k_fourier_z<T, 3, 16, true, true, GRP>));
+  FFTLS_ATTR((k_fourier_z<T, 3, 16, true, false, GRP>));
   if constexpr (!GRP) {
-    FFTLS_ATTR((k_fourier_z<T, 2, 1, false, GRP>));
-    FFTLS_ATTR((k_fourier_z<T, 2, 2, false, GRP>));
-    FFTLS_ATTR((k_fourier_z<T, 2, 4, false, GRP>));
-    FFTLS_ATTR((k_fourier_z<T, 2, 8, false, GRP>));
-    FFTLS_ATTR((k_fourier_z<T, 2, 16, false, GRP>));
+    FFTLS_ATTR((k_fourier_z<T, 2, 1, false, true, GRP>));
+    FFTLS_ATTR((k_fourier_z<T, 2, 1, false, false, GRP>));
+    FFTLS_ATTR((k_fourier_z<T, 2, 2, false, true, GRP>));
+    FFTLS_ATTR((k_fourier_z<T, 2, 2, false, false, GRP>));
+    FFTLS_ATTR((k_fourier_z<T, 2, 4, false, true, GRP>));
+    FFTLS_ATTR((k_fourier_z<T, 2, 4, false, false, GRP>));
+    FFTLS_ATTR((k_fourier_z<T, 2, 8, false, true, GRP>));
+    FFTLS_ATTR((k_fourier_z<T, 2, 8, false, false, GRP>));
+    FFTLS_ATTR((k_fourier_z<T, 2, 16, false, true, GRP>));
+    FFTLS_ATTR((k_fourier_z<T, 2, 16, false, false, GRP>));
   }
   return e;
 }

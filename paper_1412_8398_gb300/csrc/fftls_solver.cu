@@ -64,29 +64,63 @@ struct GraphCache {
   }
 };
 
+// Radices of length L's plan, first stage first: the compile-time lengths' own stages (ct_radix), else as few
+// stages as the radices allow and, among those, the smallest largest radix.  No heap allocation.
+bool radices_of(int L, int* out, int* n) {
+  if (fftls::strided_ct_length(L)) {
+    *n = fftls::ct_nst(L);
+    for (int i = 0; i < *n; ++i) out[i] = fftls::ct_radix(L, i);
+    return true;
+  }
+  if (L == 24 || L == 32) {  // tile_fft_rt's constant stages
+    *n = 2;
+    out[0] = 4;
+    out[1] = L / 4;
+    return true;
+  }
+  static const int kRadix[] = {2, 3, 4, 5, 6, 8, 9, 10, 12, 15, 16};
+  *n = 0;
+  if (L == 1) return true;
+  int best = kMaxStages + 1, best_max = 0, stack[kMaxStages];
+  // depth-first over non-increasing radices
+  struct Search {
+    int &best, &best_max, *out, *stack;
+    void go(int rem, int top, int depth) {
+      if (rem == 1) {
+        if (depth < best || (depth == best && stack[0] < best_max)) {
+          best = depth;
+          best_max = stack[0];
+          for (int i = 0; i < depth; ++i) out[i] = stack[i];
+        }
+        return;
+      }
+      if (depth + 1 > best || depth >= kMaxStages) return;
+      for (int k = (int)(sizeof(kRadix) / sizeof(kRadix[0])) - 1; k >= 0; --k) {
+        const int r = kRadix[k];
+        if (r > top || rem % r) continue;
+        stack[depth] = r;
+        go(rem / r, r, depth + 1);
+      }
+    }
+  } find{best, best_max, out, stack};
+  find.go(L, 16, 0);
+  *n = best <= kMaxStages ? best : 0;
+  return best <= kMaxStages;
+}
+
 bool factor_plan(int L, AxisPlan* p) {
   if (L < 1 || L > kMaxL) return false;
-  int n = L, twos = 0, threes = 0, fives = 0;
-  while (n % 2 == 0) { n /= 2; ++twos; }
-  while (n % 3 == 0) { n /= 3; ++threes; }
-  while (n % 5 == 0) { n /= 5; ++fives; }
-  if (n != 1) return false;
-  std::vector<int> r;
-  int n8 = twos / 3, rem = twos % 3;
-  if (rem == 1 && n8 > 0) { --n8; r.push_back(4); r.push_back(4); }
-  else if (rem == 2) r.push_back(4);
-  else if (rem == 1) r.push_back(2);
-  for (int i = 0; i < n8; ++i) r.push_back(8);
-  for (int i = 0; i < threes; ++i) r.push_back(3);
-  for (int i = 0; i < fives; ++i) r.push_back(5);
-  if ((int)r.size() > kMaxStages) return false;
+  int r[kMaxStages] = {0}, nst = 0;
+  if (!radices_of(L, r, &nst)) return false;
   p->L = L;
-  p->nst = (int)r.size();
+  p->nst = nst;
   int M = L;
   for (int i = 0; i < kMaxStages; ++i) {
-    p->radix[i] = i < p->nst ? r[i] : 1;
-    p->msize[i] = i < p->nst ? M : 1;
-    if (i < p->nst) M /= r[i];
+    p->radix[i] = i < nst ? r[i] : 1;
+    p->msize[i] = i < nst ? M : 1;
+    if (i < nst) M /= r[i];
+    p->dnb[i] = fftls::make_fastdiv(i < nst ? L / r[i] : 1);
+    p->dmr[i] = fftls::make_fastdiv(i < nst ? M : 1);
   }
   return true;
 }

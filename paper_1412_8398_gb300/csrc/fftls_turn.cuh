@@ -553,7 +553,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) k_turn_gen(const 
       }
     }
     __syncthreads();
-    tile_fft_ct<CP, NPI, true>(tile, nl, BS, a_.pl[0], tws, true);
+    tile_fft_ct<CP, NPI, true, true, false>(tile, nl, BS, a_.pl[0], tws);
     T acc[2 * NC];
 #pragma unroll
     for (int c = 0; c < 2 * NC; ++c) acc[c] = (T)0;
@@ -590,7 +590,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) k_turn_gen(const 
       if (lane == 0) wacc[warp][c] += (double)x;
     }
     __syncthreads();
-    tile_fft_ct<CP, NP, true>(tile, nl, BS, a_.pl[0], tws, false);
+    tile_fft_ct<CP, NP, true, false, false>(tile, nl, BS, a_.pl[0], tws);
     for (int idx = threadIdx.x; idx < nl * H; idx += blockDim.x) {
       const int gl = fdiv(idx, fH), k = idx - gl * H;
       const T2* r0 = tile + gl * BS + prow(__ldg(&pos[k]), 1) * CP;
