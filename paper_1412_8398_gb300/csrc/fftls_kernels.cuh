@@ -80,7 +80,8 @@ struct KTab {
 // with a_kappa = kappa0 / (kappa + kappa0), a_mu = mu0 / (mu + mu0).
 constexpr int kCoef = 8;
 
-constexpr int kSmpPar = 10;  // doubles per sample in IterArgs::smp_par
+constexpr int kGreenPar = 6;
+constexpr int kSmpPar = 8 + kGreenPar;  // doubles per sample in IterArgs::smp_par: lambda0, mu0, eps_bar[6], green_par
 
 template <typename T>
 struct IterArgs {
@@ -112,7 +113,12 @@ struct IterArgs {
   AxisPlan pl[3];
   double lam0, mu0;
   double eps_bar[6];
-  T green_cf, green_c0, inv_n;  // -1 / (N mu0), (lambda0 + mu0) / (lambda0 + 2 mu0), 1 / N
+  // Constants of Gamma' in T, worked out on the host: GB300 issues one warp-wide FP64 instruction per 16 clocks and
+  // SM, so a division and a few conversions per thread cost as much as a small FP32 pass itself (128^3, G's Fourier pass
+  // 75 -> 62 us; 100x90x75 G^C 24.5 -> 21.4 us).
+  // green_par: lambda0, mu0, -1 / (N mu0), (lambda0 + mu0) / (lambda0 + 2 mu0), 1 / (2 mu0),
+  // lambda0 / (2 mu0 (d lambda0 + 2 mu0)); inv_n: 1 / N
+  T green_par[kGreenPar], inv_n;
   Ctrl* ctrl;
   double* part_mean;   // [x1_blocks][2 nc]: sums of sigma and eps per block
   double* part_eta;    // [z blocks or eta blocks]: sums of |k*.sigma_hat|^2 per block
@@ -124,7 +130,7 @@ struct IterArgs {
                        // eta_real [3][N] floats: its real-space divergence
   // grouped launches (fftls_solve_batched): nsmp samples of one 3D geometry share a
   // launch; sample s finds its fields at these element offsets times s (null fields:
-  // offset 0) and its lambda0, mu0, eps_bar[6], green_cf, green_c0 at smp_par[kSmpPar s ..] (device memory).
+  // offset 0) and its lambda0, mu0, eps_bar[6] and the factors of Gamma' at smp_par[kSmpPar s ..] (device memory).
   // Single solves have nsmp = 1 and use the values above.
   int nsmp;
   long long st_field, st_phase, st_spec, st_coef, st_pmean, st_peta, st_pdelta, st_hist, st_d64;

@@ -52,6 +52,8 @@ __device__ __forceinline__ void at_sample(IterArgs<T>& a, int s) {
   a.mu0 = p[1];
 #pragma unroll
   for (int i = 0; i < 6; ++i) a.eps_bar[i] = p[2 + i];
+#pragma unroll
+  for (int i = 0; i < kGreenPar; ++i) a.green_par[i] = (T)p[8 + i];
 }
 
 template <int DIM> struct Comp;
@@ -66,30 +68,53 @@ template <> struct Comp<2> {
   __device__ static constexpr int J(int c) { return c < 2 ? c : 1; }
 };
 
-// Block-wide FP64 sum of W values per thread; result valid in thread 0.
+// Sums of the W <= 16 values of every lane over a warp: the total of value c is returned on the lanes from
+// c sum_lanes(W) on.  Halves of the values are exchanged and dropped on the way (16 additions for 12 values where a
+// tree per value takes 60): in FP64 an addition holds the SM's pipe for 16 clocks.
+__host__ __device__ constexpr int sum_pow2(int W) { return W <= 1 ? 1 : W <= 2 ? 2 : W <= 4 ? 4 : W <= 8 ? 8 : 16; }
+__host__ __device__ constexpr int sum_lanes(int W) { return 32 / sum_pow2(W); }
+template <int W, typename T>
+__device__ __forceinline__ T warp_sums(const T (&v)[W]) {
+  constexpr int PW = sum_pow2(W);
+  static_assert(W <= 16, "at least two lanes a value");
+  const int lane = threadIdx.x & 31;
+  T x[PW];
+#pragma unroll
+  for (int i = 0; i < PW; ++i) x[i] = i < W ? v[i < W ? i : 0] : (T)0;
+  int bit = 16;
+#pragma unroll
+  for (int h = PW / 2; h >= 1; h /= 2) {
+    const bool up = lane & bit;
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const T keep = up ? x[i + h] : x[i], give = up ? x[i] : x[i + h];
+      x[i] = keep + __shfl_xor_sync(0xffffffffu, give, bit);
+    }
+    bit /= 2;
+  }
+#pragma unroll
+  for (int o = sum_lanes(W) / 2; o >= 1; o /= 2) x[0] += __shfl_xor_sync(0xffffffffu, x[0], o);
+  return x[0];
+}
+
+// Block-wide FP64 sum of W values per thread (W <= 16, at most 32 warps); result valid in thread 0.
 template <int W>
 __device__ void block_sum(double (&v)[W]) {
   __shared__ double red[32][W];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nw = (blockDim.x + 31) >> 5;
-#pragma unroll
-  for (int i = 0; i < W; ++i) {
-    double x = v[i];
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-    v[i] = x;
-  }
+  const double t = warp_sums(v);
   __syncthreads();
-  if (lane == 0)
-#pragma unroll
-    for (int i = 0; i < W; ++i) red[warp][i] = v[i];
+  if (lane % sum_lanes(W) == 0 && lane / sum_lanes(W) < W) red[warp][lane / sum_lanes(W)] = t;
   __syncthreads();
   if (warp == 0) {
 #pragma unroll
-    for (int i = 0; i < W; ++i) {
-      double x = lane < nw ? red[lane][i] : 0.0;
-      for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-      v[i] = x;
-    }
+    for (int i = 0; i < W; ++i) v[i] = 0.0;
+    double x = 0.0;
+    if (lane < W)
+      for (int w = 0; w < nw; ++w) x += red[w][lane];
+#pragma unroll
+    for (int i = 0; i < W; ++i) v[i] = __shfl_sync(0xffffffffu, x, i);
   }
   __syncthreads();
 }
@@ -887,8 +912,8 @@ __device__ __forceinline__ void fourier_mode(const IterArgs<T>& a, int x, int y,
   const KTab<T> kt[3] = {a.kt[0][x], a.kt[1][y], a.kt[2][z]};
   const bool q0 = (x == 0 && y == 0 && z == 0);
   const T wq = (x == 0 || 2 * x == a.g.n1) ? (T)1 : (T)2;
-  const T invN = (T)(1.0 / (double)a.g.N);
-  const T mu0 = (T)a.mu0, lam0 = (T)a.lam0;
+  const T invN = a.inv_n;
+  const T mu0 = a.green_par[1], lam0 = a.green_par[0];
   T2 M[DIM][DIM];
 #pragma unroll
   for (int c = 0; c < NC; ++c) {
@@ -988,8 +1013,7 @@ __device__ __forceinline__ void fourier_mode(const IterArgs<T>& a, int x, int y,
       tr.x = (T)0; tr.y = (T)0;
 #pragma unroll
       for (int c = 0; c < DIM; ++c) { tr.x += X[c].x; tr.y += X[c].y; }
-      const T a1 = (T)(0.5 / a.mu0);
-      const T a2 = (T)(a.lam0 / (2.0 * a.mu0 * (DIM * a.lam0 + 2.0 * a.mu0)));
+      const T a1 = a.green_par[4], a2 = a.green_par[5];
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
         const bool diag = c < DIM;
@@ -1000,7 +1024,7 @@ __device__ __forceinline__ void fourier_mode(const IterArgs<T>& a, int x, int y,
 #pragma unroll
       for (int c = 0; c < NC; ++c) { E[c].x = (T)0; E[c].y = (T)0; }
     } else {
-      const T c0 = (lam0 + mu0) / (lam0 + (T)2 * mu0);
+      const T c0 = a.green_par[3];
       T2 S;
       S.x = (T)0; S.y = (T)0;
 #pragma unroll
@@ -1203,8 +1227,7 @@ __device__ __forceinline__ void k_fourier_z_body(const IterArgs<T>& a, const Axi
     const int xc = (int)threadIdx.x % W;
     if (xc < nx) {
       const T2 rx = a.rd[0][x0 + xc], ry = a.rd[1][py];
-      const T cf = (T)(-1.0 / ((double)g.N * a.mu0));
-      const T c0 = (T)((a.lam0 + a.mu0) / (a.lam0 + 2.0 * a.mu0));
+      const T cf = a.green_par[2], c0 = a.green_par[3];
       const T bxy = rx.y * ry.y, axy = rx.x * ry.y, bxay = rx.y * ry.x;
       const bool line0 = (x0 + xc == 0) && (py == 0);
       for (int pz = (int)threadIdx.x / W; pz < nl; pz += NT / W) {
@@ -1633,7 +1656,7 @@ template <typename T, int DIM>
 __global__ void k_stress(const T* eps, const uint8_t* phase, const T* coef, long long N, double* stress,
                          double* part) {
   constexpr int NC = Comp<DIM>::NC;
-  double acc[2 * NC];
+  double acc[2 * NC], ptr = 0.0;
 #pragma unroll
   for (int c = 0; c < 2 * NC; ++c) acc[c] = 0.0;
   for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < N; v += (long long)gridDim.x * blockDim.x) {
@@ -1641,15 +1664,23 @@ __global__ void k_stress(const T* eps, const uint8_t* phase, const T* coef, long
     double e[NC];
 #pragma unroll
     for (int c = 0; c < NC; ++c) e[c] = (double)eps[(long long)c * N + v];
-    double tr = e[0] + e[1] + (DIM == 3 ? e[2] : 0.0);
+    const double lam = (double)cf[0], mu2 = (double)cf[1];
+    const double tr = e[0] + e[1] + (DIM == 3 ? e[2] : 0.0);
+    if (stress) {
+      const double p = lam * tr;
+#pragma unroll
+      for (int c = 0; c < NC; ++c) stress[(long long)c * N + v] = mu2 * e[c] + (c < DIM ? p : 0.0);
+    }
+    // sum of sigma_c = sum of 2 mu e_c, plus the sum of lambda tr on the diagonal (one accumulator)
+    ptr = lam * tr + ptr;
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-      const double s = (double)cf[1] * e[c] + (c < DIM ? (double)cf[0] * tr : 0.0);
-      if (stress) stress[(long long)c * N + v] = s;
-      acc[c] += s;
+      acc[c] = mu2 * e[c] + acc[c];
       acc[NC + c] += e[c];
     }
   }
+#pragma unroll
+  for (int c = 0; c < DIM; ++c) acc[c] += ptr;
   block_sum<2 * NC>(acc);
   if (threadIdx.x == 0)
 #pragma unroll

@@ -999,9 +999,22 @@ fftls_status tune_plan(fftls_ctx* c, const Setup& S, IterArgs<T>& a, bool real_e
   return FFTLS_OK;
 }
 
-// -1 / (N mu0) and (lambda0 + mu0) / (lambda0 + 2 mu0) of the real-direction Gamma'
-double green_factor(const Setup& S, int which) {
-  return which ? (S.lam0 + S.mu0) / (S.lam0 + 2.0 * S.mu0) : -1.0 / ((double)S.g.N * S.mu0);
+// Constants of Gamma' (IterArgs::green_par)
+void green_constants(const Setup& S, double* g) {
+  const double l = S.lam0, m = S.mu0;
+  g[0] = l;
+  g[1] = m;
+  g[2] = -1.0 / ((double)S.g.N * m);
+  g[3] = (l + m) / (l + 2.0 * m);
+  g[4] = 0.5 / m;
+  g[5] = l / (2.0 * m * (S.dim * l + 2.0 * m));
+}
+template <typename T>
+void set_green(const Setup& S, IterArgs<T>& a) {
+  double g[kGreenPar];
+  green_constants(S, g);
+  for (int i = 0; i < kGreenPar; ++i) a.green_par[i] = (T)g[i];
+  a.inv_n = (T)(1.0 / (double)S.g.N);
 }
 
 template <typename T>
@@ -1049,9 +1062,7 @@ fftls_status prepare(fftls_ctx* c, const Setup& S, const fftls_problem* p, const
   a.twt = (const T2*)((const T*)tb.p + table_offset_turn(S));
   if (sizeof(T) == 4)
     for (int ax = 1; ax < 3; ++ax) a.tws[ax] = (const float4*)((const T*)tb.p + table_offset_reg(S, ax));
-  a.green_cf = (T)green_factor(S, 0);
-  a.green_c0 = (T)green_factor(S, 1);
-  a.inv_n = (T)(1.0 / (double)S.g.N);
+  set_green(S, a);
   a.eps = eps;
   a.phase = S.d_phase;
   a.specA = (T2*)c->specA.p;
@@ -1409,8 +1420,7 @@ static fftls_status solve_core(fftls_ctx* c, const fftls_problem* const* P, int 
       pi[0] = Ss[i].lam0;
       pi[1] = Ss[i].mu0;
       for (int k = 0; k < 6; ++k) pi[2 + k] = Ss[i].eps_bar[k];
-      pi[8] = green_factor(Ss[i], 0);
-      pi[9] = green_factor(Ss[i], 1);
+      green_constants(Ss[i], pi + 8);
     }
     std::vector<T> cfT(cf.begin(), cf.end());
     DevBuf& cb = Prec<T>::idx ? c->coef64 : c->coef32;
@@ -1982,6 +1992,7 @@ extern "C" fftls_status fftls_solve_noalloc(const fftls_problem* p, const fftls_
   a.lam0 = S.lam0;
   a.mu0 = S.mu0;
   for (int i = 0; i < 6; ++i) a.eps_bar[i] = S.eps_bar[i];
+  set_green(S, a);
   a.eps = eps;
   a.phase = d_phase;
   a.coef = (const double*)(base + o_coef);

@@ -323,8 +323,9 @@ template <int L, bool WILLOT>
 __device__ __forceinline__ void z_modes(const IterArgs<float>& a_, c2 (&v)[3][8], int x, int py, int pz0, int smp) {
   const double* par = a_.nsmp > 1 ? a_.smp_par + kSmpPar * smp : nullptr;
   const float2 rx = x < a_.g.H ? __ldg(&a_.rd[0][x]) : make_float2(1.f, 1.f), ry = __ldg(&a_.rd[1][py]);
-  const float cf = par ? (float)par[8] : a_.green_cf, c0 = par ? (float)par[9] : a_.green_c0;
-  const float lam0 = par ? (float)par[0] : (float)a_.lam0, mu0 = par ? (float)par[1] : (float)a_.mu0;
+  float gp[4];  // lambda0, mu0 (G^W), -1 / (N mu0), (lambda0 + mu0) / (lambda0 + 2 mu0)
+#pragma unroll
+  for (int i = 0; i < 4; ++i) gp[i] = par ? (float)par[8 + i] : a_.green_par[i];
   const float bxy = rx.y * ry.y, axy = rx.x * ry.y, bxay = rx.y * ry.x;
   const bool line0 = x == 0 && py == 0;
 #pragma unroll
@@ -338,9 +339,9 @@ __device__ __forceinline__ void z_modes(const IterArgs<float>& a_, c2 (&v)[3][8]
     }
     if (WILLOT) {
       const float2 k[3] = {rx, ry, rz};
-      green_w_mode(X, k, lam0, mu0, a_.inv_n);
+      green_w_mode(X, k, gp[0], gp[1], a_.inv_n);
     } else {
-      green_rd_mode<float>(X, axy * rz.y, bxay * rz.y, bxy * rz.x, cf, c0);
+      green_rd_mode<float>(X, axy * rz.y, bxay * rz.y, bxy * rz.x, gp[2], gp[3]);
     }
     if (line0 && pz0 + r == 0) {
 #pragma unroll

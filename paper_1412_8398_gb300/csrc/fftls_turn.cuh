@@ -17,7 +17,8 @@
 //    long chain of dependent work, so it pays only while there are enough lines for every SM (turn_reg in
 //    fftls_solver.cu: at least 64 threads per SM; FP64 128^2 in 2D, 16 threads a line: 40 us against 20).
 // What bounds it at 512^3 (FP32): 97.4 bytes per voxel, 13.1 GB per launch; 2.92 ms (4.48 TB/s, 0.66 of the
-// measured copy rate), where the two separate passes took 2.18 + 2.01 ms.  The rest is the latency of a line's
+// measured copy rate), where the two separate passes took 2.18 + 2.01 ms; 2.74 ms since the sums of <sigma>, <eps>
+// take one FP64 conversion and addition per warp and flush instead of twelve (warp_sums).  The rest is the latency of a line's
 // chain (12 synchronisations, four register transforms) at 16 warps per SM.  In FP64 the arithmetic bounds it
 // (about 250 FP64 instructions per voxel, two lanes per clock and SM): 6.78 against 3.87 + 3.11 ms at 256^3.
 // Both take the sample of a grouped launch (fftls_solve_batched) as blockIdx.y; a single solve is one
@@ -400,21 +401,17 @@ k_turn_reg(const __grid_constant__ IterArgs<T> a_) {
   const bool need_o = (upd != kUpdDirectTau && upd != kUpdCorrDirect) || a_.want_delta;  // reads the old iterate
   __shared__ double wacc[turn_threads() / 32][2 * NC];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int i = threadIdx.x; i < turn_threads() / 32 * 2 * NC; i += blockDim.x) (&wacc[0][0])[i] = 0.0;
   __syncthreads();
   T acc[2 * NC];
 #pragma unroll
   for (int c = 0; c < 2 * NC; ++c) acc[c] = (T)0;
   T dmax[2] = {(T)0, (T)0};
   int pend = 0;
+  double wsum = 0.0;  // the warp's FP64 sum of value lane / sum_lanes(2 NC)
   auto flush = [&]() {
+    wsum += (double)warp_sums(acc);
 #pragma unroll
-    for (int c = 0; c < 2 * NC; ++c) {
-      T x = acc[c];
-      for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-      if (lane == 0) wacc[warp][c] += (double)x;
-      acc[c] = (T)0;
-    }
+    for (int c = 0; c < 2 * NC; ++c) acc[c] = (T)0;
     pend = 0;
   };
   const long long step = (long long)gridDim.x * lpb;
@@ -490,6 +487,7 @@ k_turn_reg(const __grid_constant__ IterArgs<T> a_) {
     }
   }
   flush();
+  if (lane % sum_lanes(2 * NC) == 0 && lane / sum_lanes(2 * NC) < 2 * NC) wacc[warp][lane / sum_lanes(2 * NC)] = wsum;
   __syncthreads();
   if (threadIdx.x < 2 * NC) {
     double t = 0.0;
@@ -531,7 +529,10 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) k_turn_gen(const 
   const bool tauform = a_.tauform;
   __shared__ double wacc[8][2 * NC];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int i = threadIdx.x; i < 8 * 2 * NC; i += blockDim.x) (&wacc[0][0])[i] = 0.0;
+  double wsum = 0.0;  // the warp's FP64 sum of value lane / sum_lanes(2 NC)
+  T acc[2 * NC];
+#pragma unroll
+  for (int c = 0; c < 2 * NC; ++c) acc[c] = (T)0;
   T dmax[2] = {(T)0, (T)0};
   const FastDiv fL = make_fastdiv(L1), fH = make_fastdiv(H);
   for (long long l0 = (long long)blockIdx.x * G; l0 < nlines; l0 += (long long)gridDim.x * G) {
@@ -554,9 +555,6 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) k_turn_gen(const 
     }
     __syncthreads();
     tile_fft_ct<CP, NPI, true, true, false>(tile, nl, BS, a_.pl[0], tws);
-    T acc[2 * NC];
-#pragma unroll
-    for (int c = 0; c < 2 * NC; ++c) acc[c] = (T)0;
     for (int idx = threadIdx.x; idx < nl * L1; idx += blockDim.x) {
       const int gl = fdiv(idx, fL), x = idx - gl * L1;
       const long long vox = (l0 + gl) * (long long)L1 + x;
@@ -583,11 +581,10 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) k_turn_gen(const 
         row[p] = cmk<T2>(c0 < NC ? out[c0 % NC] : s[c0 % NC], c1 >= nout ? (T)0 : (c1 < NC ? out[c1 % NC] : s[c1 % NC]));
       }
     }
+    if (sizeof(T) == 4) {
+      wsum += (double)warp_sums(acc);
 #pragma unroll
-    for (int c = 0; c < 2 * NC; ++c) {
-      T x = acc[c];
-      for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-      if (lane == 0) wacc[warp][c] += (double)x;
+      for (int c = 0; c < 2 * NC; ++c) acc[c] = (T)0;
     }
     __syncthreads();
     tile_fft_ct<CP, NP, true, false, false>(tile, nl, BS, a_.pl[0], tws);
@@ -613,6 +610,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) k_turn_gen(const 
     }
     __syncthreads();
   }
+  if (sizeof(T) == 8) wsum = (double)warp_sums(acc);
+  if (lane % sum_lanes(2 * NC) == 0 && lane / sum_lanes(2 * NC) < 2 * NC) wacc[warp][lane / sum_lanes(2 * NC)] = wsum;
   __syncthreads();
   if (threadIdx.x < 2 * NC) {
     double t = 0.0;
