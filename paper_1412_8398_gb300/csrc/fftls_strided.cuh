@@ -445,9 +445,9 @@ __device__ __forceinline__ bool tma_tile_load(unsigned char* tile, float4* tws, 
                   AX == 1 ? other : r, smp, bar);
     }
   }
-  reg_tables<L>(tws, tw);
   __syncthreads();
-  if (!*flag) return false;
+  if (!*flag) return false;  // before anything else: a stopped solve's passes still come to the end of their beat
+  reg_tables<L>(tws, tw);
   bool done = false;
   for (long long k = 0; k < kBulkWaitRounds && !done; ++k) done = mbar_try_wait(bar, 0);
   if (__syncthreads_or(!done)) {
