@@ -94,7 +94,7 @@ struct IterArgs {
   int corr;          // 1: correction phase (zero mean mode, eta adds d64)
   int want_delta;    // inverse x1 pass computes max |d eps|, |d sigma|
   int write_d64;     // store the FP64 iterate's divergence (FP32) for a later correction phase
-  int eta_real;      // 1: eta from the real-space divergence stencil (G^C/W/R, 3D, k_eta_stencil);
+  int eta_real;      // 1: eta from the real-space divergence stencil (G^C/W/R, k_eta_stencil, k_eta_2d);
                      //    the forward transform then carries tau only
   int tauform;       // 1: the transformed field is tau (mean mode = eps_bar); 0: sigma
   T* eps;            // n_c x N (the iterate, or the correction delta)
@@ -191,8 +191,12 @@ __host__ __device__ constexpr int turn_tw_count(int L) {
 // Launchers (fftls_kernels.cu).  All return cudaGetLastError().
 template <typename T> cudaError_t launch_fwd_x(const IterArgs<T>& a, cudaStream_t s);
 template <typename T> cudaError_t launch_eta_stencil(const IterArgs<T>& a, cudaStream_t s);
-// tile of the real-space eta kernel (x1 columns x x2 rows) and its threads
-constexpr int kEtaTileX = 64, kEtaTileY = 8;
+// tile of the real-space eta kernel (x1 columns x x2 rows): 64 columns, or 32 where those cover n1 with fewer
+// columns to spare (n1 <= 32, 75, 90, 96, ...) and in 2D
+constexpr int kEtaTileY = 8;
+__host__ __device__ constexpr int eta_tile_x(int dim, int n1) {
+  return dim == 2 || (n1 + 31) / 32 * 32 < (n1 + 63) / 64 * 64 ? 32 : 64;
+}
 template <typename T> cudaError_t launch_mid_y(const IterArgs<T>& a, bool inv, cudaStream_t s);
 template <typename T> cudaError_t launch_fourier_z(const IterArgs<T>& a, cudaStream_t s);
 template <typename T> cudaError_t launch_reduce_eta(const IterArgs<T>& a, cudaStream_t s);

@@ -672,7 +672,7 @@ __global__ void __launch_bounds__(256, 4) k_fwd_x_staged(const __grid_constant__
 }
 
 // ---------------------------------------------------------------------------
-// E (3D, G^C / G^W / G^R): the equilibrium norm from the real-space divergence
+// E (G^C / G^W / G^R): the equilibrium norm from the real-space divergence
 // ---------------------------------------------------------------------------
 // For the finite-difference operators the divergence k*(q).sigma_hat(q) is the
 // transform of a stencil applied to sigma on the grid (eq. mul1, wil071 and the
@@ -688,9 +688,9 @@ __global__ void __launch_bounds__(256, 4) k_fwd_x_staged(const __grid_constant__
 //   R: div(z) = U(z) + V(z) + [U - V](z-1)             (backward differences averaged
 //                                                       over the other two axes)
 //   C: div(z-1) = U(z-1) + (V(z) - V(z-2)) / 2         (centred differences)
-constexpr int kEX = kEtaTileX, kEY = kEtaTileY, kEThreads = 256;
-constexpr int kERows = kEThreads / kEX;     // thread rows; each thread owns kEY / kERows voxels
-constexpr int kEOwn = kEY / kERows;
+// (EX = kEX columns, 64 or 32: a 24^3 grid in FP64, where every warp-wide instruction holds the FP64 pipe whether its
+// lanes have a voxel or not, took 50 us on 64-column tiles and slabs of four planes, 17 us on 32 columns and slabs chosen from one plane up.)
+constexpr int kEY = kEtaTileY, kEThreads = 256;
 
 template <typename T>
 __device__ __forceinline__ void sigma_of(const T* __restrict__ eps, const uint8_t* __restrict__ phase,
@@ -711,9 +711,11 @@ __device__ __forceinline__ int wrap_index(int i, int n) {
   return i;
 }
 
-template <typename T, bool CEN>
+template <typename T, bool CEN, int kEX>
 __device__ __forceinline__ void k_eta_stencil_body(const IterArgs<T>& a, const AxisPlan* pl) {
   if (!__syncthreads_or(a.ctrl->state == kRunning)) return;  // block-uniform: a strided pass beside it may stop the solve
+  constexpr int kERows = kEThreads / kEX;  // thread rows; each thread owns kEY / kERows voxels
+  constexpr int kEOwn = kEY / kERows;
   const Geom g = a.g;
   const int n1 = g.n1, n2 = g.n2, n3 = g.n3;
   const long long N = g.N;
@@ -835,15 +837,66 @@ __device__ __forceinline__ void k_eta_stencil_body(const IterArgs<T>& a, const A
 }
 
 // GRP: a grouped launch (fftls_solve_batched), every block working on its sample's view
-template <typename T, bool CEN, bool GRP>
+template <typename T, bool CEN, int EX, bool GRP>
 __global__ void __launch_bounds__(kEThreads) k_eta_stencil(const __grid_constant__ IterArgs<T> a_) {
   if constexpr (GRP) {
     IterArgs<T> a = a_;
     at_sample(a, blockIdx.y);
-    k_eta_stencil_body<T, CEN>(a, a_.pl);
+    k_eta_stencil_body<T, CEN, EX>(a, a_.pl);
   } else {
-    k_eta_stencil_body<T, CEN>(a_, a_.pl);
+    k_eta_stencil_body<T, CEN, EX>(a_, a_.pl);
   }
+}
+
+// The same in 2D (one voxel per thread, 32 x 8 tiles): sigma on the tile and its halo in shared memory, then
+//   W: backward differences; R: backward differences averaged over the other axis (the symbol of eq. wil14 up to its
+//   phase); C: centred differences.
+// With eta from here only tau is transformed (the Fourier-space norm needed sigma's transforms too: 512^2 FP64,
+// G^R accelerated, 235 -> 224 us per iteration; 128^2, direct, 39 -> 30 us).
+template <typename T>
+__global__ void __launch_bounds__(kEThreads) k_eta_2d(const __grid_constant__ IterArgs<T> a) {
+  if (!__syncthreads_or(a.ctrl->state == kRunning)) return;
+  constexpr int EX = 32, SX = EX + 2, SY = kEY + 2;
+  __shared__ T S[3][SY][SX];
+  const int n1 = a.g.n1, n2 = a.g.n2;
+  const long long N = a.g.N;
+  const int ntx = (n1 + EX - 1) / EX;
+  const int x0 = (int)(blockIdx.x % ntx) * EX, y0 = (int)(blockIdx.x / ntx) * kEY;
+  for (int e = threadIdx.x; e < SY * SX; e += kEThreads) {
+    const int r = e / SX, c = e - r * SX;
+    const long long v = (long long)wrap_index(y0 - 1 + r, n2) * n1 + wrap_index(x0 - 1 + c, n1);
+    const T* cf = a.coef + (int)a.phase[v] * kCoef;
+    const T e0 = a.eps[v], e1 = a.eps[N + v], e2 = a.eps[2 * N + v];
+    const T p = cf[0] * (e0 + e1);
+    S[0][r][c] = cf[1] * e0 + p;
+    S[1][r][c] = cf[1] * e1 + p;
+    S[2][r][c] = cf[1] * e2;
+  }
+  __syncthreads();
+  const int tx = threadIdx.x % EX, ty = threadIdx.x / EX;
+  const int x = x0 + tx, y = y0 + ty;
+  T se = (T)0;
+  if (x < n1 && y < n2) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const T(*P)[SX] = S[j == 0 ? 0 : 2];  // sigma_1j: its x1 difference
+      const T(*Q)[SX] = S[j == 0 ? 2 : 1];  // sigma_2j: its x2 difference
+      const int r = ty + 1, c = tx + 1;
+      T d;
+      if (a.green == kCentered) d = (T)0.5 * ((P[r][c + 1] - P[r][c - 1]) + (Q[r + 1][c] - Q[r - 1][c]));
+      else if (a.green == kWillot) d = (P[r][c] - P[r][c - 1]) + (Q[r][c] - Q[r - 1][c]);
+      else
+        d = (T)0.5 * (((P[r][c] - P[r][c - 1]) + (P[r - 1][c] - P[r - 1][c - 1])) +
+                      ((Q[r][c] - Q[r - 1][c]) + (Q[r][c - 1] - Q[r - 1][c - 1])));
+      const long long v = (long long)y * n1 + x;
+      if (a.write_d64) reinterpret_cast<float*>(a.d64)[(long long)j * N + v] = (float)d;
+      if (a.corr) d += (T)reinterpret_cast<const float*>(a.d64)[(long long)j * N + v];
+      se += d * d;
+    }
+  }
+  double e1[1] = {(double)se * (double)N};
+  block_sum<1>(e1);
+  if (threadIdx.x == 0) a.part_eta[blockIdx.x] = e1[0];
 }
 
 // ---------------------------------------------------------------------------
@@ -1166,6 +1219,22 @@ __device__ __forceinline__ void green_rd_mode(T2 (&X)[6], T k0, T k1, T k2, T cf
   X[5].y = h * (fk[0] * U[1].y + fk[1] * U[0].y);
 }
 
+// The same in 2D (three components 11, 22, 12).
+template <typename T, typename T2>
+__device__ __forceinline__ void green_rd_mode(T2 (&X)[3], T k0, T k1, T cf, T c0) {
+  const T K2 = k0 * k0 + k1 * k1;
+  const T iK2 = K2 > (T)0 ? recip_pos(K2) : (T)0;
+  const T2 V0 = cmk<T2>(X[0].x * k0 + X[2].x * k1, X[0].y * k0 + X[2].y * k1);
+  const T2 V1 = cmk<T2>(X[2].x * k0 + X[1].x * k1, X[2].y * k0 + X[1].y * k1);
+  const T hs = c0 * iK2;
+  const T Sx = (k0 * V0.x + k1 * V1.x) * hs, Sy = (k0 * V0.y + k1 * V1.y) * hs;
+  const T2 U0 = cmk<T2>(V0.x - k0 * Sx, V0.y - k0 * Sy), U1 = cmk<T2>(V1.x - k1 * Sx, V1.y - k1 * Sy);
+  const T f = cf * iK2, f0 = f * k0, f1 = f * k1, h = (T)0.5;
+  X[0] = cmk<T2>(f0 * U0.x, f0 * U0.y);
+  X[1] = cmk<T2>(f1 * U1.x, f1 * U1.y);
+  X[2] = cmk<T2>(h * (f0 * U1.x + f1 * U0.x), h * (f0 * U1.y + f1 * U0.y));
+}
+
 // Six complex values of one mode between registers and the tile (16-byte accesses;
 // a mode starts on a 48-byte (float) or 96-byte (double) boundary).
 __device__ __forceinline__ void load_mode6(const float2* p, float2 (&X)[6]) {
@@ -1191,7 +1260,7 @@ __device__ __forceinline__ void store_mode6(double2* p, const double2 (&X)[6]) {
   for (int i = 0; i < 6; ++i) p[i] = X[i];
 }
 
-// FAST: 3D G^C / G^R with eta from the real-space stencil (only tau is
+// FAST: G^C / G^R with eta from the real-space stencil (only tau is
 // transformed, no eta here): the modes take green_rd_mode with the per-axis
 // factors of rd (by storage position), kr_1 = a_1 b_2 b_3, kr_2 = b_1 a_2 b_3,
 // kr_3 = b_1 b_2 a_3.  Otherwise the general fourier_mode.
@@ -1223,24 +1292,41 @@ __device__ __forceinline__ void k_fourier_z_body(const IterArgs<T>& a, const Axi
   tile_fft_strided<C, NT, false, false, CT>(tile, pl[AX], tws);
   T eta_acc = (T)0;
   if constexpr (FAST) {
-    static_assert(DIM == 3 && NT % W == 0, "fast Fourier pass: 3D, whole modes per thread");
+    static_assert(NT % W == 0, "fast Fourier pass: whole modes per thread");
     const int xc = (int)threadIdx.x % W;
     if (xc < nx) {
-      const T2 rx = a.rd[0][x0 + xc], ry = a.rd[1][py];
+      const T2 rx = a.rd[0][x0 + xc];
       const T cf = a.green_par[2], c0 = a.green_par[3];
-      const T bxy = rx.y * ry.y, axy = rx.x * ry.y, bxay = rx.y * ry.x;
       const bool line0 = (x0 + xc == 0) && (py == 0);
+      T bxy = (T)0, axy = (T)0, bxay = (T)0;
+      if constexpr (DIM == 3) {
+        const T2 ry = a.rd[1][py];
+        bxy = rx.y * ry.y;
+        axy = rx.x * ry.y;
+        bxay = rx.y * ry.x;
+      }
       for (int pz = (int)threadIdx.x / W; pz < nl; pz += NT / W) {
-        const T2 rz = __ldg(&a.rd[2][pz]);
+        const T2 rz = __ldg(&a.rd[AX][pz]);
         T2* mp = tile + pz * C + xc * NC;
-        T2 X[6];
-        load_mode6(mp, X);
-        green_rd_mode<T>(X, axy * rz.y, bxay * rz.y, bxy * rz.x, cf, c0);
+        T2 X[NC];
+        if constexpr (DIM == 3) {
+          load_mode6(mp, X);
+          green_rd_mode<T>(X, axy * rz.y, bxay * rz.y, bxy * rz.x, cf, c0);
+        } else {
+#pragma unroll
+          for (int c = 0; c < NC; ++c) X[c] = mp[c];
+          green_rd_mode<T>(X, rx.x * rz.y, rx.y * rz.x, cf, c0);
+        }
         if (line0 && pz == 0) {
 #pragma unroll
-          for (int c = 0; c < 6; ++c) { X[c].x = a.corr ? (T)0 : (T)a.eps_bar[c]; X[c].y = (T)0; }
+          for (int c = 0; c < NC; ++c) { X[c].x = a.corr ? (T)0 : (T)a.eps_bar[c]; X[c].y = (T)0; }
         }
-        store_mode6(mp, X);
+        if constexpr (DIM == 3) {
+          store_mode6(mp, X);
+        } else {
+#pragma unroll
+          for (int c = 0; c < NC; ++c) mp[c] = X[c];
+        }
       }
     }
   } else {
@@ -1747,8 +1833,16 @@ cudaError_t launch_fwd_x_t(const IterArgs<T>& a, cudaStream_t s) {
 template <typename T, bool GRP>
 cudaError_t launch_eta_stencil_t(const IterArgs<T>& a, cudaStream_t s) {
   const dim3 grid(a.e_blocks, GRP ? a.nsmp : 1);
-  if (a.green == kCentered) k_eta_stencil<T, true, GRP><<<grid, kEThreads, a.e_smem, s>>>(a);
-  else k_eta_stencil<T, false, GRP><<<grid, kEThreads, a.e_smem, s>>>(a);
+  if constexpr (!GRP)
+    if (a.dim == 2) {
+      k_eta_2d<T><<<grid, kEThreads, 0, s>>>(a);
+      return cudaGetLastError();
+    }
+  const bool cen = a.green == kCentered;
+  if (eta_tile_x(a.dim, a.g.n1) == 32)
+    (cen ? k_eta_stencil<T, true, 32, GRP> : k_eta_stencil<T, false, 32, GRP>)<<<grid, kEThreads, a.e_smem, s>>>(a);
+  else
+    (cen ? k_eta_stencil<T, true, 64, GRP> : k_eta_stencil<T, false, 64, GRP>)<<<grid, kEThreads, a.e_smem, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -1774,10 +1868,10 @@ cudaError_t launch_mid_y_t(const IterArgs<T>& a, bool inv, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// The fast Fourier pass serves 3D G^C / G^R when eta comes from the real-space stencil.
+// The fast Fourier pass serves G^C / G^R when eta comes from the real-space stencil.
 template <typename T>
 bool fourier_fast(const IterArgs<T>& a) {
-  return a.dim == 3 && a.eta_real && (a.green == kCentered || a.green == kRotated);
+  return a.eta_real && (a.green == kCentered || a.green == kRotated);
 }
 
 template <typename T, bool GRP>
@@ -1799,7 +1893,8 @@ cudaError_t launch_fourier_z_t(const IterArgs<T>& a, cudaStream_t s) {
     if (fourier_fast(a)) { FFTLS_FZ_W(3, true) }
     else { FFTLS_FZ_W(3, false) }
   } else if constexpr (!GRP) {
-    FFTLS_FZ_W(2, false)
+    if (fourier_fast(a)) { FFTLS_FZ_W(2, true) }
+    else { FFTLS_FZ_W(2, false) }
   } else {
     return cudaErrorInvalidValue;
   }
@@ -1907,15 +2002,25 @@ cudaError_t set_attrs_z_t(size_t smax) {
   FFTLS_ATTR((k_fourier_z<T, 3, 16, true, false, GRP>));
   if constexpr (!GRP) {
     FFTLS_ATTR((k_fourier_z<T, 2, 1, false, true, GRP>));
+    FFTLS_ATTR((k_fourier_z<T, 2, 1, true, true, GRP>));
     FFTLS_ATTR((k_fourier_z<T, 2, 1, false, false, GRP>));
+    FFTLS_ATTR((k_fourier_z<T, 2, 1, true, false, GRP>));
     FFTLS_ATTR((k_fourier_z<T, 2, 2, false, true, GRP>));
+    FFTLS_ATTR((k_fourier_z<T, 2, 2, true, true, GRP>));
     FFTLS_ATTR((k_fourier_z<T, 2, 2, false, false, GRP>));
+    FFTLS_ATTR((k_fourier_z<T, 2, 2, true, false, GRP>));
     FFTLS_ATTR((k_fourier_z<T, 2, 4, false, true, GRP>));
+    FFTLS_ATTR((k_fourier_z<T, 2, 4, true, true, GRP>));
     FFTLS_ATTR((k_fourier_z<T, 2, 4, false, false, GRP>));
+    FFTLS_ATTR((k_fourier_z<T, 2, 4, true, false, GRP>));
     FFTLS_ATTR((k_fourier_z<T, 2, 8, false, true, GRP>));
+    FFTLS_ATTR((k_fourier_z<T, 2, 8, true, true, GRP>));
     FFTLS_ATTR((k_fourier_z<T, 2, 8, false, false, GRP>));
+    FFTLS_ATTR((k_fourier_z<T, 2, 8, true, false, GRP>));
     FFTLS_ATTR((k_fourier_z<T, 2, 16, false, true, GRP>));
+    FFTLS_ATTR((k_fourier_z<T, 2, 16, true, true, GRP>));
     FFTLS_ATTR((k_fourier_z<T, 2, 16, false, false, GRP>));
+    FFTLS_ATTR((k_fourier_z<T, 2, 16, true, false, GRP>));
   }
   return e;
 }
@@ -1923,8 +2028,10 @@ cudaError_t set_attrs_z_t(size_t smax) {
 template <typename T, bool GRP>
 cudaError_t set_attrs_x_t(size_t smax) {
   cudaError_t e = cudaSuccess;
-  FFTLS_ATTR((k_eta_stencil<T, true, GRP>));
-  FFTLS_ATTR((k_eta_stencil<T, false, GRP>));
+  FFTLS_ATTR((k_eta_stencil<T, true, 32, GRP>));
+  FFTLS_ATTR((k_eta_stencil<T, false, 32, GRP>));
+  FFTLS_ATTR((k_eta_stencil<T, true, 64, GRP>));
+  FFTLS_ATTR((k_eta_stencil<T, false, 64, GRP>));
   FFTLS_ATTR((k_fwd_x<T, 3, true, 1, GRP>));
   FFTLS_ATTR((k_fwd_x<T, 3, false, 1, GRP>));
   if constexpr (!GRP) {

@@ -512,7 +512,8 @@ PlanGeom plan_geom(const Setup& S, size_t cb, bool real_eta) {
   G.line1 = (size_t)padded_rows(S.g.n1) * odd_up(real_eta ? (nc + 1) / 2 : nc) * cb;
   G.line5 = (size_t)padded_rows(S.g.n1) * odd_up((nc + 1) / 2) * cb;
   G.nlines = (long long)S.g.n2 * S.g.n3;
-  G.tiles = (long long)((S.g.n1 + kEtaTileX - 1) / kEtaTileX) * ((S.g.n2 + kEtaTileY - 1) / kEtaTileY);
+  const int ex = eta_tile_x(S.dim, S.g.n1);
+  G.tiles = (long long)((S.g.n1 + ex - 1) / ex) * ((S.g.n2 + kEtaTileY - 1) / kEtaTileY);
   return G;
 }
 
@@ -547,7 +548,7 @@ TilePlan default_plan(const Setup& S, size_t cb, bool real_eta) {
   P.z_w = pick_w(S.g.n3);
   const long long want_slabs = std::max<long long>(1, (8LL * S.num_sms + G.tiles - 1) / G.tiles);
   int Z = (int)((S.g.n3 + want_slabs - 1) / want_slabs);
-  P.e_planes = std::max(std::min(Z, 32), std::min(4, S.g.n3));
+  P.e_planes = std::max(1, std::min(Z, 32));
   return P;
 }
 
@@ -613,7 +614,7 @@ bool apply_plan(const Setup& S, IterArgs<T>& a, bool real_eta, const TilePlan& P
     const int Z = std::max(1, std::min(P.e_planes, g.n3));
     a.e_planes = Z;
     a.e_blocks = (int)(G.tiles * ((g.n3 + Z - 1) / Z));
-    a.e_smem = (size_t)2 * 6 * (kEtaTileY + 2) * (kEtaTileX + 2) * sizeof(T);
+    a.e_smem = (size_t)2 * 6 * (kEtaTileY + 2) * (eta_tile_x(S.dim, g.n1) + 2) * sizeof(T);
   }
   return true;
 }
@@ -764,7 +765,7 @@ struct Runner {
     return read_ctrl();
   }
 
-  // eta of the current iterate without the transforms (3D G^C/G^W/G^R): the real-space
+  // eta of the current iterate without the transforms (G^C/G^W/G^R): the real-space
   // stencil, the means of sigma and eps, and the reduction's stop decision (no update).
   fftls_status certify(const Ctrl* init) {
     fftls_status st;
@@ -1008,8 +1009,8 @@ fftls_status tune_plan(fftls_ctx* c, const Setup& S, IterArgs<T>& a, bool real_e
     apply_plan<T>(S, a, real_eta, P);
   }
   a.eps = keep.eps;
-  if (real_eta)
-    search(&TilePlan::e_planes, {4, 8, 16, 32, 64},
+  if (real_eta && S.dim == 3)
+    search(&TilePlan::e_planes, {1, 2, 4, 8, 16, 32, 64},
            [](const IterArgs<T>& x, cudaStream_t st) { return launch_eta_stencil<T>(x, st); });
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
@@ -1050,7 +1051,7 @@ fftls_status prepare(fftls_ctx* c, const Setup& S, const fftls_problem* p, const
   a.lam0 = S.lam0;
   a.mu0 = S.mu0;
   for (int i = 0; i < 6; ++i) a.eps_bar[i] = S.eps_bar[i];
-  const bool real_eta = S.dim == 3 && S.green != kMS;
+  const bool real_eta = S.green != kMS;
   const PlanKey key{Prec<T>::idx, S.g.n1, S.g.n2, S.g.n3, S.dim, S.green, real_eta ? 1 : 0};
   int cached = -1;
   for (size_t i = 0; i < c->plans.size(); ++i)
@@ -1146,7 +1147,7 @@ fftls_status fftls_tile_plans(const fftls_ctx* c, int* rows, int* count) {
     const PlanKey& k = c->plans[i].first;
     const TilePlan& P = c->plans[i].second;
     const int row[FFTLS_PLAN_FIELDS] = {k.prec,     k.n1,  k.n2,  k.n3, k.green, P.x1_lines, P.x1_vb,
-                                        P.x5_lines, P.y_w, P.z_w, k.real_eta ? P.e_planes : 0, P.tuned,
+                                        P.x5_lines, P.y_w, P.z_w, k.real_eta && k.dim == 3 ? std::min(P.e_planes, k.n3) : 0, P.tuned,
                                         P.y_thr,    P.z_thr, P.x5_vb};
     memcpy(rows + (size_t)i * FFTLS_PLAN_FIELDS, row, sizeof(row));
   }
@@ -1183,8 +1184,8 @@ fftls_status fftls_set_tile_plans(fftls_ctx* c, const int* rows, int count) {
     // a row names the grid, not the dimension: it serves the 3D problem on it and, with n3 = 1, the 2D one
     for (int dim = 2; dim <= 3; ++dim) {
       if (dim == 2 && n3 != 1) continue;
-      const bool real_eta = dim == 3 && green != kMS;
-      if (real_eta && P.e_planes < 1) continue;
+      const bool real_eta = green != kMS;
+      if (real_eta && dim == 3 && P.e_planes < 1) continue;
       add.push_back({PlanKey{prec, n1, n2, n3, dim, green, real_eta ? 1 : 0}, P});
     }
   }
@@ -1432,7 +1433,7 @@ static fftls_status solve_core(fftls_ctx* c, const fftls_problem* const* P, int 
     }
   }
   const bool direct = p->scheme == FFTLS_DIRECT;
-  // G^C / G^W / G^R in 3D take eta from the real-space stencil and transform tau
+  // G^C / G^W / G^R take eta from the real-space stencil and transform tau
   // only (tau form for both schemes); otherwise AS transforms tau and sigma and
   // DS uses the sigma form while its iterate is compatible.
   auto upd_of = [&](bool er) { return direct ? (er ? (int)kUpdDirectTau : (int)kUpdDirectSig) : (int)kUpdAccel; };
