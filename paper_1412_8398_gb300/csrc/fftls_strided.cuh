@@ -534,16 +534,21 @@ __host__ __device__ constexpr size_t strided_tma_smem() {
   return (size_t)L * W * 48 + (size_t)strided_reg_tw(L, ct_nst(L)) * 16;
 }
 
+// Blocks per SM of k_z_tma: three of 128 threads at 512, whose 164 registers without a spill are worth more than a
+// fourth block (1.557 against 1.597 ms); four at the shorter lengths (128^3 31.1 -> 28.9 us, 256^3 188 -> 185 us).
+__host__ __device__ constexpr int strided_tma_blocks_z(int L, int W) {
+  return (L == 512 ? 384 : 512) / strided_reg_threads_z(L, W) > 12 ? 12 : (L == 512 ? 384 : 512) / strided_reg_threads_z(L, W);
+}
 template <int L, int W, bool WILLOT>
-__global__ void __launch_bounds__(strided_reg_threads_z(L, W), 384 / strided_reg_threads_z(L, W) > 12 ? 12 : 384 / strided_reg_threads_z(L, W))
+__global__ void __launch_bounds__(strided_reg_threads_z(L, W), strided_tma_blocks_z(L, W))
 k_z_tma(const __grid_constant__ IterArgs<float> a_) {
   constexpr int C = 3 * W;
   constexpr int SL = ct_nst(L) - 1;
-  extern __shared__ __align__(128) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_tile[];  // the copy engine's boxes start on 128 bytes
   __shared__ __align__(8) uint64_t bar_word;
   __shared__ int flag;
-  unsigned char* tile = smem_raw;
-  float4* tws = reinterpret_cast<float4*>(smem_raw + (size_t)L * W * 48);
+  unsigned char* tile = smem_tile;
+  float4* tws = reinterpret_cast<float4*>(smem_tile + (size_t)L * W * 48);
   const int smp = blockIdx.z, py = blockIdx.y, x0 = blockIdx.x * W;
   if (!tma_tile_load<L, W, 2>(tile, tws, a_.tws[2], &a_.tm[2], x0, py, smp, a_.ctrl + smp, &bar_word, &flag)) return;
   const int w = threadIdx.x % W, a = threadIdx.x / W;
@@ -592,11 +597,11 @@ k_y_tma(const __grid_constant__ IterArgs<float> a_, int kinds) {
   constexpr int SL = ct_nst(L) - 1;
   static_assert(NT % C == 0, "whole rows of units per turn");
   constexpr int DA = NT / C;
-  extern __shared__ __align__(128) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_tile[];  // the copy engine's boxes start on 128 bytes
   __shared__ __align__(8) uint64_t bar_word;
   __shared__ int flag;
-  unsigned char* tile = smem_raw;
-  float4* tws = reinterpret_cast<float4*>(smem_raw + (size_t)L * W * 48);
+  unsigned char* tile = smem_tile;
+  float4* tws = reinterpret_cast<float4*>(smem_tile + (size_t)L * W * 48);
   const int smp = blockIdx.z / kinds, kind = blockIdx.z % kinds, pz = blockIdx.y, x0 = blockIdx.x * W;
   const CUtensorMap* map = &a_.tm[kind];
   if (!tma_tile_load<L, W, 1>(tile, tws, a_.tws[1], map, x0, pz, smp, a_.ctrl + smp, &bar_word, &flag)) return;
@@ -767,19 +772,17 @@ cudaError_t launch_z_reg(const IterArgs<float>& a, cudaStream_t s) {
     const cudaError_t e = spectrum_map(&b.tm[2], a, a.specA, W, a.g.n3 < 256 ? a.g.n3 : 256, 2);
     if (e != cudaSuccess) return e;
 #define F(LV, WV)                                                                                                  \
-  if (a.g.n3 == LV && W == WV) {                                                                                   \
-    if (will) k_z_tma<LV, WV, true><<<grid, strided_reg_threads_z(LV, WV), strided_tma_smem<LV, WV>(), s>>>(b);    \
-    else k_z_tma<LV, WV, false><<<grid, strided_reg_threads_z(LV, WV), strided_tma_smem<LV, WV>(), s>>>(b);        \
-  }
+  if (a.g.n3 == LV && W == WV)                                                                                     \
+    (will ? k_z_tma<LV, WV, true> : k_z_tma<LV, WV, false>)<<<grid, strided_reg_threads_z(LV, WV),                 \
+                                                              strided_tma_smem<LV, WV>(), s>>>(b);
     FFTLS_TMA_CASES(F)
 #undef F
     return cudaGetLastError();
   }
 #define F(LV, WV)                                                                                                  \
-  if (a.g.n3 == LV && W == WV) {                                                                                   \
-    if (will) k_z_reg<LV, WV, true><<<grid, strided_reg_threads_z(LV, WV), strided_reg_smem(LV, WV), s>>>(a);      \
-    else k_z_reg<LV, WV, false><<<grid, strided_reg_threads_z(LV, WV), strided_reg_smem(LV, WV), s>>>(a);          \
-  }
+  if (a.g.n3 == LV && W == WV)                                                                                     \
+    (will ? k_z_reg<LV, WV, true> : k_z_reg<LV, WV, false>)<<<grid, strided_reg_threads_z(LV, WV),                 \
+                                                              strided_reg_smem(LV, WV), s>>>(a);
   FFTLS_REG_CASES(F)
 #undef F
   return cudaGetLastError();
