@@ -226,6 +226,9 @@ fftls_status fftls_solve_batched(fftls_ctx* ctx, const fftls_problem* probs, int
  * the x3 pass (0: chosen from the tile size), how the inverse x1 pass reads eps
  * (1: loaded by the threads, 0: staged in shared memory by bulk copies, FP32)}.  Copies min(*count, held) rows into
  * `rows` (may be NULL when *count is 0) and returns the number held in *count.
+ * The lines of the inverse x1 pass are also those of the x1 turn's tiles; the register kernels of
+ * the lengths 64, 128, 256, 512 use the widths as far as they have them; in 2D the Fourier pass runs
+ * along x2 with the x2 pass's width.
  * The paper has no counterpart (an implementation detail of the GPU path). */
 #define FFTLS_PLAN_FIELDS 15
 fftls_status fftls_tile_plans(const fftls_ctx* ctx, int* rows, int* count);

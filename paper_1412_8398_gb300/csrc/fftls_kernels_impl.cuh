@@ -5,19 +5,18 @@
 // _y32/_y64 (x2 pass) and _z32/_z64 (x3 + Fourier pass) each instantiate their
 // share, so the library's kernels compile in parallel.
 //
-// One iteration is five passes over the fields in HBM:
-//   K1 fwd_x     : sigma = C(x):eps (and tau = sigma - C0:eps) per voxel,
-//                  fused with the x1 real-to-half-complex transform; FP64 sums
-//                  of <sigma>, <eps>                          (eq. ls, a1)
-//   K2 mid_y     : transform along x2 (forward)
-//   K3 fourier_z : transform along x3, then per mode the equilibrium norm
-//                  |k* . sigma_hat|^2 and e_hat = -G'(k):x_hat, the mean mode,
-//                  the 1/N of eq. ft, then the inverse transform along x3
-//                                                             (eq. discFour2, criterion)
-//   R  reduce_eta: eta, <sigma> history and the stop decision (one block)
-//   K2 mid_y     : inverse transform along x2
-//   K5 inv_x     : half-complex-to-real along x1 fused with the scheme update
-//                  (eq. ds or eq. as), optional max |delta| for the max-delta stop
+// One iteration in steady state (fftls_solver.cu, turn_iteration):
+//   K2 mid_y     : transform along x2 (forward), 3D
+//   K3 fourier_z : transform along x3 (2D: x2), then per mode e_hat = -G'(k):x_hat, the
+//                  mean mode, the 1/N of eq. ft (and for G the equilibrium norm
+//                  |k* . sigma_hat|^2), then the inverse transform   (eq. discFour2)
+//   K2 mid_y     : inverse transform along x2, 3D
+//   E  eta       : the equilibrium norm from the real-space divergence (G^C / G^W / G^R)
+//   R  reduce_eta: eta, <sigma> history and the stop decision (one block; criterion)
+//   turn         : inverse x1 transform, scheme update, law of the new iterate, forward
+//                  x1 transform (fftls_turn.cuh)                     (eq. ls, ds, as)
+// The FP32 lengths 64..512 of K2 and K3 have register kernels (fftls_strided.cuh).  The
+// separate x1 passes start a run (fwd_x) and take the ladder's FP64 defect (fwd_x, inv_x).
 // The half spectrum is array-of-structures [x3 pos][x2 pos][x1][component]: a
 // strided pass reads rows of W modes x n_c components (192 contiguous bytes in
 // FP32 with W = 4, n_c = 6).  Along x2 and x3 the spectrum is kept in the

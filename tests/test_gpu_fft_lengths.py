@@ -69,3 +69,22 @@ def test_turn_lines(solver, n1, n2, n3, green, scheme):
 def test_register_passes(solver, n, green):
     for shape in ((n, 3, 18), (3, n, 18), (n, n if n < 256 else 64, 5)):
         _check(solver, shape, green, "AS", "fp32")
+
+
+@pytest.mark.parametrize("shape", [(64, 128, 18), (128, 64, 10), (20, 64, 64)])
+@pytest.mark.parametrize("green", ["R", "W", "MS"])
+def test_grouped_register_kernels(solver, shape, green):
+    """Grouped samples (the sample is a dimension of the tensor maps, and of the turn's grid) give bit for bit what
+    each gives alone."""
+    rng = np.random.default_rng(7)
+    batch = []
+    for i in range(3):
+        lam, mu = MS.binary_moduli(4.0 + 5 * i, 3)
+        batch.append({"phase": (rng.random(shape) < 0.3).astype(np.uint8), "lam": lam, "mu": mu,
+                      "eps_bar": np.diag([1.0, 0.2 * i, -0.1]), "green": green, "scheme": "AS"})
+    kw = dict(tol=1e-6, max_iter=60, precision="fp32_refine64", autotune=False)
+    res, _ = solver.solve_batched(batch, concurrency=1, want_strain=True, **kw)
+    for b, r in zip(batch, res):
+        q = solver.solve(b["phase"], b["lam"], b["mu"], b["eps_bar"], green, "AS", raise_on_error=False, **kw)
+        assert (r.status, r.iterations) == (q.status, q.iterations)
+        assert np.array_equal(r.strain, q.strain)
