@@ -29,6 +29,7 @@ enum Update : int {
   kUpdResidual = 3,   // r <- e - eps (eps unchanged)    (defect of the current iterate)
   kUpdCorrDirect = 4, // delta <- r + e                  (correction, direct scheme)
   kUpdCorrAccel = 5,  // delta <- delta + 2 M (r + e - delta) (correction, accelerated)
+  kUpdForward = 6,    // x1 turn (register variant) without its inverse transform and update: the spectrum of the iterate
 };
 
 // Mutable solver control block (device memory, written by the host between

@@ -378,7 +378,8 @@ __device__ __forceinline__ void line_unpack(T2* spec, const T2 (&v)[NP][8], T2* 
 // x1 lines per block of k_turn_reg (host and device): 128 threads
 __host__ __device__ constexpr int turn_threads() { return 128; }
 
-template <typename T, int DIM, int L>
+// FWD (kUpdForward): no inverse transform and no update, the spectrum of the iterate as it is
+template <typename T, int DIM, int L, bool FWD>
 __global__ void __launch_bounds__(turn_threads(), sizeof(T) == 4 ? 4 : 2)
 k_turn_reg(const __grid_constant__ IterArgs<T> a_) {
   typedef typename Cplx<T>::type T2;
@@ -426,17 +427,17 @@ k_turn_reg(const __grid_constant__ IterArgs<T> a_) {
       if (a < (L + 127) / 128) asm volatile("prefetch.global.L2 [%0];" ::"l"(V.phase + ln * L + a * 128));
     }
     T2 v[NP][8];
-    line_pack<T, L, NC, NP>(V.specA + ln * H * NC, v, buf, a, line);
+    if (!FWD) line_pack<T, L, NC, NP>(V.specA + ln * H * NC, v, buf, a, line);
     {  // the next line's spectrum
       const long long nx = ln + step;
-      if (nx < nlines) {
+      if (!FWD && nx < nlines) {
         const char* base = reinterpret_cast<const char*>(V.specA + nx * H * NC);
         constexpr int bytes = (L / 2 + 1) * NC * (int)sizeof(T2);
         for (int off = a * 128; off < bytes; off += P::M * 128)
           asm volatile("prefetch.global.L2 [%0];" ::"l"(base + off));
       }
     }
-    line_inverse<T, L, NP>(v, buf, tw, a, line);
+    if (!FWD) line_inverse<T, L, NP>(v, buf, tw, a, line);
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
       const long long vox = ln * L + a + P::M * r;
@@ -444,15 +445,20 @@ k_turn_reg(const __grid_constant__ IterArgs<T> a_) {
       load_coef(V.coef + (int)V.phase[vox] * kCoef, cf);
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
-        e[c] = (c & 1) ? v[c / 2][r].y : v[c / 2][r].x;
+        if (!FWD) e[c] = (c & 1) ? v[c / 2][r].y : v[c / 2][r].x;
         o[c] = need_o ? V.eps[(long long)c * N + vox] : (T)0;
       }
-      turn_update<T, DIM>(upd, e, o, V.rfield + vox, N, cf, n);
+      if constexpr (FWD) {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) n[c] = o[c];
+      } else {
+        turn_update<T, DIM>(upd, e, o, V.rfield + vox, N, cf, n);
+      }
       turn_law<T, DIM>(n, cf, tauform, s, out);
       if (active) {
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
-          V.eps[(long long)c * N + vox] = n[c];
+          if (!FWD) V.eps[(long long)c * N + vox] = n[c];
           acc[c] += s[c];
           acc[NC + c] += n[c];
         }
@@ -635,11 +641,12 @@ template <typename T, int DIM>
 cudaError_t launch_turn_d(const IterArgs<T>& a, cudaStream_t s) {
   const dim3 grid(a.x_blocks, a.nsmp > 1 ? a.nsmp : 1);
   if (a.t_reg) {
+    const bool fwd = a.update == kUpdForward;
     switch (a.g.n1) {
-      case 64: k_turn_reg<T, DIM, 64><<<grid, a.t_threads, a.t_smem, s>>>(a); break;
-      case 128: k_turn_reg<T, DIM, 128><<<grid, a.t_threads, a.t_smem, s>>>(a); break;
-      case 256: k_turn_reg<T, DIM, 256><<<grid, a.t_threads, a.t_smem, s>>>(a); break;
-      default: k_turn_reg<T, DIM, 512><<<grid, a.t_threads, a.t_smem, s>>>(a); break;
+      case 64: (fwd ? k_turn_reg<T, DIM, 64, true> : k_turn_reg<T, DIM, 64, false>)<<<grid, a.t_threads, a.t_smem, s>>>(a); break;
+      case 128: (fwd ? k_turn_reg<T, DIM, 128, true> : k_turn_reg<T, DIM, 128, false>)<<<grid, a.t_threads, a.t_smem, s>>>(a); break;
+      case 256: (fwd ? k_turn_reg<T, DIM, 256, true> : k_turn_reg<T, DIM, 256, false>)<<<grid, a.t_threads, a.t_smem, s>>>(a); break;
+      default: (fwd ? k_turn_reg<T, DIM, 512, true> : k_turn_reg<T, DIM, 512, false>)<<<grid, a.t_threads, a.t_smem, s>>>(a); break;
     }
   } else if (a.dual) {
     k_turn_gen<T, DIM, true><<<grid, a.t_threads, a.t_smem, s>>>(a);
@@ -659,14 +666,22 @@ cudaError_t set_attrs_turn(size_t smax) {
   auto set = [&](const void* f) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smax);
   };
-  set((const void*)k_turn_reg<T, 3, 64>);
-  set((const void*)k_turn_reg<T, 3, 128>);
-  set((const void*)k_turn_reg<T, 3, 256>);
-  set((const void*)k_turn_reg<T, 3, 512>);
-  set((const void*)k_turn_reg<T, 2, 64>);
-  set((const void*)k_turn_reg<T, 2, 128>);
-  set((const void*)k_turn_reg<T, 2, 256>);
-  set((const void*)k_turn_reg<T, 2, 512>);
+  set((const void*)k_turn_reg<T, 3, 64, false>);
+  set((const void*)k_turn_reg<T, 3, 64, true>);
+  set((const void*)k_turn_reg<T, 3, 128, false>);
+  set((const void*)k_turn_reg<T, 3, 128, true>);
+  set((const void*)k_turn_reg<T, 3, 256, false>);
+  set((const void*)k_turn_reg<T, 3, 256, true>);
+  set((const void*)k_turn_reg<T, 3, 512, false>);
+  set((const void*)k_turn_reg<T, 3, 512, true>);
+  set((const void*)k_turn_reg<T, 2, 64, false>);
+  set((const void*)k_turn_reg<T, 2, 64, true>);
+  set((const void*)k_turn_reg<T, 2, 128, false>);
+  set((const void*)k_turn_reg<T, 2, 128, true>);
+  set((const void*)k_turn_reg<T, 2, 256, false>);
+  set((const void*)k_turn_reg<T, 2, 256, true>);
+  set((const void*)k_turn_reg<T, 2, 512, false>);
+  set((const void*)k_turn_reg<T, 2, 512, true>);
   set((const void*)k_turn_gen<T, 3, true>);
   set((const void*)k_turn_gen<T, 3, false>);
   set((const void*)k_turn_gen<T, 2, true>);
