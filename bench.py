@@ -683,10 +683,11 @@ def run_warmstart(args, rank, local, world):
 
 
 def run_x1_sweep(args, rank, local):
-    """The forward x1 pass (k_fwd_x) on the workload (--n) for lines per batch 1..8 and the load variants
+    """The forward x1 pass (k_fwd_x) on the workload's recipe for lines per batch 1..8 and the load variants
     (voxels per thread loaded together 1, 2, 4; 0 = the batch staged in shared memory by bulk copies),
     the other passes on the tuned schedule: CUDA-event ms per launch over 8 FP32 iterations (the
-    solver's profile mode), best of two rounds.  Rank 0 only."""
+    solver's profile mode), best of two rounds.  The grid is --n, or 480 for the lengths whose first
+    spectrum comes from the x1 turn instead.  Rank 0 only."""
     import numpy as np
     import torch
     from paper_1412_8398_gb300 import build, fftls
@@ -695,7 +696,8 @@ def run_x1_sweep(args, rank, local):
         return
     build.build()
     torch.cuda.set_device(local)
-    ph, lam, mu, _ = workload(args.n)
+    n = 480 if args.n in (64, 128, 256, 512) else args.n
+    ph, lam, mu, _ = workload(n)
     dph = torch.from_numpy(ph).cuda()
     eb = np.diag([1.0, 0.0, 0.0])
     s = fftls.Solver(local)
@@ -718,7 +720,7 @@ def run_x1_sweep(args, rank, local):
                     res[key] = min(res.get(key, float("inf")), v[0] / v[1])
     finally:
         s.close()
-    print(json.dumps({"metric": f"k_fwd_x ms per launch at {args.n}^3 FP32 by (lines per batch, voxels per load; "
+    print(json.dumps({"metric": f"k_fwd_x ms per launch at {n}^3 FP32 by (lines per batch, voxels per load; "
                                 "0 = staged by bulk copies)", "tuned": {k: base[k] for k in ("x1_lines", "x1_vb")},
                       "ms": res}), flush=True)
 
